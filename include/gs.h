@@ -443,7 +443,8 @@ gs_status gs_centre_rois(gs_context *ctx, const uint8_t *cls, int width, int hei
  *         at tile 8, 2 or 4 at tile 16, 2, 4 or 8 at tile 32.
  *   batch 32, 64, 128 or 256 surfel records per shared-memory stage.
  * Every configuration produces the same images bit for bit; they differ in
- * speed only. The default is {16, 4, 128} ({32, 8, 128} when min_tile = 32).
+ * speed only. (The rasterizer may use another block shape or a shorter stage
+ * where it is faster; 16- and 32-pixel tiles are blended in 16-pixel squares.) The default is {16, 4, 128} ({32, 8, 128} when min_tile = 32).
  * Returns GS_ERR_BAD_ARG for any other value. */
 typedef struct {
   int tile, pix, batch;

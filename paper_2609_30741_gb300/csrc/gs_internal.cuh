@@ -283,6 +283,7 @@ struct RasterFrame {
   int rshift, rtiles_x;     // > 0: the tile lists are those of a grid 1 << rshift times coarser
                             // (rtiles_x columns), each raster tile reads its parent's list
   const uint32_t *n_items;  // device count of the listed tiles
+  int split;                // 1: every tile is four work items, its quadrants (set by launch_raster)
   float *rgb, *depth, *trans;  // [3][H][W], [H][W] (or null), [H][W] (or null)
   uint8_t *cls;             // class map: written pixels get kClsRender, or null
   unsigned long long *winit;  // warp buffer cleared (no sample) at every written pixel, or null
