@@ -18,12 +18,9 @@ int g_pdl = 1;
 namespace {
 
 constexpr size_t kAlign = 256;
-// widest image: the binning keeps 8 warps x 4 tile rows x 2 counters per tile
-// column in shared memory (128 KB at 512 tile columns, the limit)
+// widest image: the binning keeps 8 warps x 4 tile rows x 1 counter per tile
+// column in shared memory (64 KB at kMaxTileCols), and per tile row 8 counters
 constexpr int kMaxWidth = 8192;
-constexpr int kMaxTileCols = 512;
-
-
 
 struct Carver {
   char *base;
@@ -68,9 +65,12 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   ws.bin_nch = bin_chunks(lim.max_surfels);
   const size_t table = tiles * ws.bin_nch;
   ws.cnt_bin = c.take<uint32_t>(lim.keep_intermediates ? N : 1);
-  // a band-list entry covers at least one span of its surfel, so the spans'
-  // capacity bounds the entries too
-  for (int e = 0; e < 2; ++e) ws.band_pool_cap[e] = (uint32_t)(Ie[e] < 8 * N ? Ie[e] + 1024 : 8 * N + 1024);
+  // the row-list entries are the spans, but for an ROI binning's rows without a
+  // masked tile, and one more for each of the few spans with two ranges
+  for (int e = 0; e < 2; ++e) {
+    ws.row_pool_cap[e] = (uint32_t)(Ie[e] + Ie[e] / 8 + 1024);
+    ws.band_cap[e] = (uint32_t)(Ie[e] < 8 * N ? Ie[e] + 1024 : 8 * N + 1024);
+  }
   const size_t rs_words = radix_status_words(N);
   for (int e = 0; e < 2; ++e) {  // one binning scratch per eye
     BinScratch &b = ws.bin[e];
@@ -81,8 +81,8 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
     b.ival = c.take<uint32_t>(Ie[e]);
     b.ikey = c.take<uint32_t>(lim.keep_intermediates ? Ie[e] : 1);
     b.bin_table = c.take<uint4>(table);
-    b.band_pool = reinterpret_cast<BandEntry *>(c.take<char>(kBandEntryBytes * ws.band_pool_cap[e]));
-    b.band_lists = c.take<uint2>(band_list_words(lim.max_surfels, (int)rty));  // the binning runs on the raster grid
+    b.row_pool = reinterpret_cast<RowEntry *>(c.take<char>(kRowEntryBytes * ws.row_pool_cap[e]));
+    b.row_lists = c.take<uint2>(row_list_words(lim.max_surfels, (int)rty));  // the binning runs on the raster grid
     b.bin_offs = c.take<uint32_t>(table);
     b.ranges = c.take<uint2>(tiles);
     b.rmask = c.take<uint8_t>(tiles);
@@ -104,7 +104,7 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   ws.strip_mask = c.take<uint8_t>(tiles);
   ws.strip_rgb = c.take<float>(reuse ? 3 * P : 1);
   for (int e = 0; e < 2; ++e) {
-    ws.row_off[e] = c.take<uint32_t>(N);
+    ws.info[e] = c.take<uint4>(N);
     ws.spans[e] = c.take<uint2>(Ie[e]);
   }
   ws.warpbuf = c.take<unsigned long long>(stereo ? P : 1);
@@ -169,6 +169,7 @@ __global__ void reset_counters_kernel(Counters *c) {
     c->n_sort[0] = c->n_sort[1] = 0;
     c->n_rows[0] = c->n_rows[1] = 0;
     c->n_band[0] = c->n_band[1] = 0;
+    c->n_entries[0] = c->n_entries[1] = 0;
     c->n_union = 0;
     c->n_items[0] = c->n_items[1] = 0;
     c->dmin_bits = 0x7f800000u;
@@ -398,7 +399,7 @@ gs_status gs_context_create(gs_context **out, const gs_limits *lim, void *worksp
     return GS_ERR_WORKSPACE;
   }
   const int msh = min_tshift(*lim);
-  cudaError_t e = prepare_binning((lim->max_width + (1 << msh) - 1) >> msh);
+  cudaError_t e = prepare_binning((lim->max_width + (1 << msh) - 1) >> msh, (lim->max_height + (1 << msh) - 1) >> msh);
   if (e == cudaSuccess) e = prepare_repair();
   if (e == cudaSuccess) e = prepare_reproject();
   for (int k = 0; k < 2 && e == cudaSuccess; ++k) {

@@ -8,6 +8,8 @@
 
 namespace gs {
 
+// tile columns of the widest rasterizer grid a context may ask for
+constexpr int kMaxTileCols = 512;
 // ROI grid: the ROI generator aligns its rectangles to 16x16 tiles (Sec. 3.5),
 // whatever tile edge the rasterizer runs with (8, 16 or 32 pixels).
 constexpr int kTile = 16;
@@ -66,7 +68,8 @@ struct Counters {
   uint32_t n_rects;      // centre components found
   uint32_t n_sort[2];    // instances actually binned per eye (capacity-clamped)
   uint32_t n_rows[2];    // (surfel, tile row) spans per eye
-  uint32_t n_band[2];    // (surfel, band) list entries of the last binning per eye
+  uint32_t n_band[2];    // (surfel, band of 4 tile rows) pairs of the last binning per eye
+  uint32_t n_entries[2]; // row list entries of the last binning per eye
   uint32_t n_union;      // surfels in the dominant binning's depth order (both eyes' visible set)
   uint32_t n_items[2];   // rasterizer tiles listed by the last masked binning per eye
   uint32_t prev_range[2];// float bits of the last measured depth range (reused by depth_mode 2)
@@ -94,8 +97,8 @@ struct Record {
 struct BinScratch {
   uint32_t *dkey[2], *dval[2];  // depth sort double buffers
   uint4 *bin_table;             // [tile][chunk] per-warp instance counts (8 x 16 bits)
-  struct BandEntry *band_pool;  // (surfel, band) entries of every warp's lists
-  uint2 *band_lists;            // [chunk][band][warp]: first entry, entries
+  struct RowEntry *row_pool;    // (surfel, row range) entries of every warp's lists
+  uint2 *row_lists;             // [chunk][row][warp]: first entry, entries
   uint32_t *bin_offs;           // their tile-major exclusive scan
   uint32_t *ival;               // surfel id per instance, grouped by tile, depth order inside
   uint32_t *ikey;               // tile id per instance (keep_intermediates)
@@ -125,12 +128,13 @@ struct Workspace {
   uint32_t *zkey[2];            // float bits of the centre depth per surfel and eye
   uint32_t *cnt_bin;            // tiles each surfel reaches in the last binning (keep_intermediates)
   uint32_t *uval;               // depth-ordered union of both eyes' binned surfels (dominant keys)
-  uint32_t band_pool_cap[2];     // per eye
+  uint32_t row_pool_cap[2];     // entries of row_pool, per eye
+  uint32_t band_cap[2];         // bound on an eye's (surfel, band of 4 tile rows) pairs
   BinScratch bin[2];            // per eye
   uint8_t *tile_mask;           // ROI mask on the 16-pixel grid
   uint8_t *strip_mask;          // edge-strip tiles of a reused depth range (16-pixel grid)
   float *strip_rgb;             // [3][pixels] the affiliated eye's strip tiles, rendered ahead
-  uint32_t *row_off[2];         // per surfel and eye: slot of its first rectangle row in spans
+  uint4 *info[2];               // per surfel and eye: rectangle, slot of its first row in spans, flags
   uint2 *spans[2];              // per (surfel, tile row): tile ranges [a0, a1] u [c0, c1], 4 x 16 bits
   // scans outside the binning (centre ROIs, repair tile lists) use bin[0]'s scratch
   unsigned long long *warpbuf;
@@ -220,9 +224,9 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
 // shared-memory opt-in of its kernel for the widest image.
 uint32_t bin_warp_surfels(int max_surfels);
 uint32_t bin_chunks(int max_surfels);
-size_t band_list_words(int max_surfels, int max_tiles_y);
-constexpr size_t kBandEntryBytes = 12;
-cudaError_t prepare_binning(int max_tiles_x);
+size_t row_list_words(int max_surfels, int max_tiles_y);
+constexpr size_t kRowEntryBytes = 8;
+cudaError_t prepare_binning(int max_tiles_x, int max_tiles_y);
 // ---- learned repair network ----
 constexpr int kRepairParams = 39908;
 struct RepairBatch {
