@@ -59,8 +59,8 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
     ws.bounds[e] = c.take<float4>(N);  // the rasterizer's per-warp culling reads them
     ws.cnt[e] = c.take<uint32_t>(N);
     ws.zkey[e] = c.take<uint32_t>(N);
+    ws.vis[e] = c.take<uint32_t>((N + 31) / 32);
   }
-  ws.uval = c.take<uint32_t>(N);
   ws.bin_warp_surfels = bin_warp_surfels(lim.max_surfels);
   ws.bin_nch = bin_chunks(lim.max_surfels);
   const size_t table = tiles * ws.bin_nch;
@@ -78,6 +78,7 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
       b.dkey[k] = c.take<uint32_t>(N);
       b.dval[k] = c.take<uint32_t>(N);
     }
+    b.bits = c.take<uint32_t>((N + 31) / 32);
     b.ival = c.take<uint32_t>(Ie[e]);
     b.ikey = c.take<uint32_t>(lim.keep_intermediates ? Ie[e] : 1);
     b.bin_table = c.take<uint4>(table);
@@ -159,26 +160,6 @@ bool limits_ok(const gs_limits *lim) {
          lim->max_width <= kMaxWidth && lim->max_height <= kMaxWidth &&
          (lim->min_tile == 0 || lim->min_tile == 8 || lim->min_tile == 16 || lim->min_tile == 32) &&
          ((lim->max_width + (1 << min_tshift(*lim)) - 1) >> min_tshift(*lim)) <= kMaxTileCols;
-}
-
-__global__ void reset_counters_kernel(Counters *c) {
-  griddep_wait();
-  if (threadIdx.x == 0) {
-    c->n_vis[0] = c->n_vis[1] = 0;
-    c->n_inst[0] = c->n_inst[1] = 0;
-    c->n_sort[0] = c->n_sort[1] = 0;
-    c->n_rows[0] = c->n_rows[1] = 0;
-    c->n_band[0] = c->n_band[1] = 0;
-    c->n_entries[0] = c->n_entries[1] = 0;
-    c->n_union = 0;
-    c->n_items[0] = c->n_items[1] = 0;
-    c->dmin_bits = 0x7f800000u;
-    c->dmax_bits = 0u;
-    c->n_rects = 0;
-    c->n_centre = 0;
-    c->pairs[0] = c->pairs[1] = 0ull;
-    c->contrib[0] = c->contrib[1] = 0ull;
-  }
 }
 
 }  // namespace
@@ -338,12 +319,6 @@ cudaError_t copy_optional(gs_context *ctx, const gs_outputs *out, int W, int H) 
            (const uint8_t *)ctx->ws.cls, out->cls_aff, npix, (const int4 *)ctx->ws.rects,
            reinterpret_cast<int4 *>(out->roi_rects), (uint32_t)ctx->lim.max_rects, (const Counters *)ctx->ws.ctr,
            out->roi_count, (const int32_t *)ctx->ws.widths, out->edge_widths);
-  GS_LAUNCHED(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reset_counters(Counters *c, cudaStream_t s) {
-  launch_k(reset_counters_kernel, 1, 32, 0, s, c);
   GS_LAUNCHED(1);
   return cudaGetLastError();
 }
@@ -518,7 +493,7 @@ static void mark(gs_context *ctx, int slot) {
 
 // One eye through the persistent rasterizer (a table of one frame).
 // The stream and events on which a binning computes its row spans beside its
-// compaction and depth sort (created on first use); null if they cannot be.
+// depth order (created on first use); null if they cannot be.
 static const SideRows *side_rows(gs_context *ctx) {
   static thread_local SideRows r;
   if (!ctx->rows || !ctx->ev_rfork || !ctx->ev_rjoin) {
@@ -569,8 +544,7 @@ static gs_status render_eye_full(gs_context *ctx, const gs_scene *scene, int eye
 static gs_status begin_call(gs_context *ctx, const gs_scene *scene, const PoseArgs &pa) {
   cudaStream_t s = ctx->stream;
   ctx->nmarks = 0;
-  cudaError_t e = launch_reset_counters(ctx->ws.ctr, s);
-  if (e == cudaSuccess) e = launch_setup_cams(pa, ctx->ws.cams, s);
+  cudaError_t e = launch_setup_cams(pa, ctx->ws.cams, ctx->ws.ctr, s);
   if (e != cudaSuccess) return cuda_fail(e);
   mark(ctx, 0);  // the first stage is the preprocessing kernel alone
   e = launch_preprocess(*scene, ctx->ws, pa.neyes, pa.W, pa.H, s);
@@ -663,12 +637,13 @@ static gs_status run_graph(gs_context *ctx, int kind, const void *key, size_t ke
   } else {
     PoseArgs arg = pa;
     CamBlock *cams = ctx->ws.cams;
-    void *args[2] = {(void *)&arg, (void *)&cams};
+    Counters *ctr = ctx->ws.ctr;
+    void *args[3] = {(void *)&arg, (void *)&cams, (void *)&ctr};
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof(kp));
     kp.func = const_cast<void *>(setup_cams_kernel_ptr());
     kp.gridDim = dim3(1);
-    kp.blockDim = dim3(32);
+    kp.blockDim = dim3(kSetupThreads);
     kp.kernelParams = args;
     if (cudaGraphExecKernelNodeSetParams(g.exec, g.setup_node, &kp) != cudaSuccess) return cuda_fail(cudaGetLastError());
   }

@@ -136,8 +136,7 @@ static gs_status enqueue_batch(gs_batch *b, const gs_frame *frames, int n, const
   for (int f = 0; f < n; ++f) {
     gs_context *ctx = b->slot[f];
     cudaStream_t s = ctx->stream;
-    BTRY(launch_reset_counters(ctx->ws.ctr, s));
-    BTRY(launch_setup_cams(g[f].pa, ctx->ws.cams, s));
+    BTRY(launch_setup_cams(g[f].pa, ctx->ws.cams, ctx->ws.ctr, s));
     BTRY(launch_preprocess(*frames[f].scene, ctx->ws, 2, g[f].W, g[f].H, s));
     BTRY(launch_binning(ctx->ws, 0, frames[f].scene->n, g[f].tx, g[f].ty, nullptr, s,
                         g[f].pa.parallel ? kOrderUnion : kOrderOwn));
@@ -210,8 +209,7 @@ static gs_status enqueue_mono(gs_batch *b, const gs_mono_frame *frames, int n, c
   for (int f = 0; f < n; ++f) {
     gs_context *ctx = b->slot[f];
     cudaStream_t s = ctx->stream;
-    BTRY(launch_reset_counters(ctx->ws.ctr, s));
-    BTRY(launch_setup_cams(g[f].pa, ctx->ws.cams, s));
+    BTRY(launch_setup_cams(g[f].pa, ctx->ws.cams, ctx->ws.ctr, s));
     BTRY(launch_preprocess(*frames[f].scene, ctx->ws, 1, g[f].W, g[f].H, s));
     BTRY(launch_binning(ctx->ws, 0, frames[f].scene->n, g[f].tx, g[f].ty, nullptr, s, kOrderOwn));
   }
@@ -311,12 +309,13 @@ static gs_status batch_run(gs_batch *b, int kind, const KeyBuilder &kb, const Fr
     for (int f = 0; f < n; ++f) {
       PoseArgs arg = g[f].pa;
       CamBlock *cams = b->slot[f]->ws.cams;
-      void *args[2] = {(void *)&arg, (void *)&cams};
+      Counters *ctr = b->slot[f]->ws.ctr;
+      void *args[3] = {(void *)&arg, (void *)&cams, (void *)&ctr};
       cudaKernelNodeParams kp;
       memset(&kp, 0, sizeof(kp));
       kp.func = const_cast<void *>(setup_cams_kernel_ptr());
       kp.gridDim = dim3(1);
-      kp.blockDim = dim3(32);
+      kp.blockDim = dim3(kSetupThreads);
       kp.kernelParams = args;
       if (cudaGraphExecKernelNodeSetParams(gr.exec, gr.setup[f], &kp) != cudaSuccess) return BFAIL(cudaGetLastError());
     }

@@ -26,14 +26,14 @@
 // low-pass disc.
 //
 // Pipeline per eye (all counts stay on the device):
-//   1. compact the surfels with a non-empty rectangle (reaching an ROI tile when
-//      a mask is given) -> (depth bits, id)
-//   2. tile ranges of every rectangle row of those surfels (rows_kernel)
-//   3. radix sort over the 32 depth bits
-//   4. per chunk and warp, depth-ordered lists of every tile row's ranges
-//   5. per-(tile, chunk) counts (bin_count_kernel)
-//   6. tile-major scan of the counts -> run offsets, tile ranges
-//   7. placement of every surfel id (bin_place_kernel)
+//   1. tile ranges of every rectangle row (rows_kernel); an ROI binning also
+//      selects the surfels whose rectangle holds an ROI tile
+//   2. radix sort of the selected surfels over the 32 depth bits, or the dominant
+//      eye's order filtered
+//   3. per chunk and warp, depth-ordered lists of every tile row's ranges
+//   4. per-(tile, chunk) counts (bin_count_kernel)
+//   5. tile-major scan of the counts -> run offsets, tile ranges
+//   6. placement of every surfel id (bin_place_kernel)
 #include <mutex>
 
 #include "gs_conic.cuh"
@@ -95,8 +95,10 @@ __device__ __forceinline__ void row_ranges(const Conic &q, const float4 r0, int 
 __global__ void __launch_bounds__(1024) mask_sat_kernel(uint8_t *mask, int tiles_x, int tiles_y,
                                                         uint32_t *__restrict__ sat, const uint8_t *__restrict__ roi16,
                                                         int rtx, int rty, int tshift, uint16_t *__restrict__ clip,
-                                                        uint32_t *__restrict__ list16) {
+                                                        uint32_t *__restrict__ list16,
+                                                        uint32_t *__restrict__ n_rows) {
   griddep_wait();
+  if (threadIdx.x == 0) *n_rows = 0u;  // the row spans of this binning follow
   constexpr int kSatSmem = 12000;
   __shared__ uint32_t s_sat[kSatSmem];
   __shared__ uint32_t s_n16;
@@ -223,37 +225,40 @@ constexpr uint32_t kInfoBinned = 1u, kInfoSplit = 2u;
 // with one atomic, and then computes the rows 32 at a time, one per lane, so no
 // lane idles while another walks a large surfel. info[i] collects what the row
 // lists need of surfel i in one 16-byte record, because they gather it at random
-// in depth order: the rectangle, the slot of its first row and flags. An ROI binning keeps of each range only the
-// part from its first to its last masked tile. The grid strides over the
-// surfels, so a small grid can run beside other kernels; without ids the
-// candidates are all surfels by id, and with the ROI's summed-area table a
-// surfel whose rectangle holds no ROI tile is skipped (the compaction's test),
-// so the spans need neither the compaction nor the depth order.
-__global__ void __launch_bounds__(256) rows_kernel(const uint32_t *__restrict__ ids, const uint32_t *n_ptr,
-                                                   uint32_t n_max, const float4 *__restrict__ rec,
-                                                   const ushort4 *__restrict__ rect, const uint32_t *__restrict__ cnt,
+// in depth order: the rectangle, the slot of its first row and flags. An ROI
+// binning keeps of each range only the part from its first to its last masked
+// tile, skips the surfels whose rectangle holds no ROI tile, and marks the others
+// in `bits`, the selection its depth order is taken from: the test then runs once
+// per surfel in id order (coalesced), and the order filters a bit mask. The grid
+// strides over the surfels, so a small grid can run beside other kernels.
+__global__ void __launch_bounds__(256) rows_kernel(uint32_t n, const float4 *__restrict__ rec,
+                                                   const ushort4 *__restrict__ rect,
+                                                   const uint32_t *__restrict__ vis,
                                                    const CamBlock *__restrict__ cams, int eye, int prim,
                                                    uint4 *__restrict__ info, uint2 *__restrict__ spans,
                                                    uint32_t cap, uint32_t *__restrict__ n_rows,
                                                    uint32_t *__restrict__ status, const uint16_t *__restrict__ clip,
                                                    int clip_tiles_x, int clip_tiles_y,
-                                                   const uint32_t *__restrict__ sat, int mark_all) {
+                                                   const uint32_t *__restrict__ sat, uint32_t *__restrict__ bits) {
   griddep_wait();
   const int lane = threadIdx.x & 31;
-  const uint32_t n = load_n(n_ptr, n_max);
   const int W = cams->eye[eye].W, H = cams->eye[eye].H, tshift = cams->eye[eye].tshift;
   const uint32_t stride = gridDim.x * blockDim.x;  // a multiple of 32: j0 stays warp-aligned
   for (uint32_t j0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; j0 < n; j0 += stride) {  // warp-uniform
-  const uint32_t j = j0 + (uint32_t)lane;
-  const uint32_t i = j < n ? (ids ? ids[j] : j) : 0u;  // the surfels being binned
+  const uint32_t i = j0 + (uint32_t)lane;
   int nr = 0, ry = 0, rx0 = 0, rx1 = -1;
   Conic q{};
   float cx = 0.f, cy = 0.f;
-  bool bin = j < n && cnt[i] > 0u;
+  bool bin = (vis[j0 >> 5] >> lane) & 1u;
   ushort4 rc = make_ushort4(0, 0, 0, 0);
   if (bin) {
     rc = rect[i];
     if (sat) bin = sat_any(sat, clip_tiles_x, rc.y, rc.w, rc.x, rc.z);  // the binning's ROI test
+  }
+  if (bits) {
+    const uint32_t m = __ballot_sync(0xffffffffu, bin);
+    if (lane == 0) bits[j0 >> 5] = m;
+    if (!m) continue;  // warp-uniform; the lists hold none of these
   }
   if (bin) {
     nr = (int)rc.w - (int)rc.y + 1;
@@ -325,44 +330,26 @@ __global__ void __launch_bounds__(256) rows_kernel(const uint32_t *__restrict__ 
     }
     split |= __reduce_or_sync(0xffffffffu, two ? 1u << k : 0u);
   }
-  if (j < n && (bin || mark_all))  // without mark_all the lists hold no unbinned surfel
+  if (i < n && (bin || !bits))  // with a selection of its own the lists hold no unbinned surfel
     info[i] = make_uint4((uint32_t)rc.x | ((uint32_t)rc.y << 16), (uint32_t)rc.z | ((uint32_t)rc.w << 16),
                          base + (uint32_t)(incl - nr),
                          (bin ? kInfoBinned : 0u) | (((split >> lane) & 1u) ? kInfoSplit : 0u));
   }
 }
 
-// ---------------------------------------------------------------- compaction
+// ---------------------------------------------------------------- depth order
 // A surfel enters the depth sort when its bounding rectangle is not empty and,
-// for an ROI binning, when that rectangle holds at least one ROI tile. The union
+// for an ROI binning, when that rectangle holds at least one ROI tile; the union
 // variant (dominant eye of a parallel two-eye call) takes every surfel either
 // eye bins.
-struct VisibleLoad {
-  const uint32_t *cnt;
-  const uint32_t *cnt_other;  // union with the other eye's binned set, or null
-  const ushort4 *rect;
-  const uint32_t *sat;        // summed-area table of the ROI mask, or null
-  int tiles_x;
-  __device__ uint32_t operator()(uint32_t i) const {
-    // the count and the rectangle are loaded together (one memory round trip)
-    const bool mine = cnt[i] > 0u;
-    const ushort4 rc = sat ? rect[i] : make_ushort4(0, 0, 0, 0);
-    if (cnt_other) return (mine || cnt_other[i] > 0u) ? 1u : 0u;
-    if (!mine) return 0u;
-    if (!sat) return 1u;
-    return sat_any(sat, tiles_x, rc.y, rc.w, rc.x, rc.z) ? 1u : 0u;
-  }
-};
-
-// What the compaction's last CTA sets up for the rest of a binning: the binned
-// count, cleared row-span, list and tile-list counters, the chunks holding
-// binned surfels and the size of the (tile, chunk) table scan over them.
+// What the depth order's last CTA sets up for the rest of a binning: the binned
+// count, cleared list and tile-list counters, the chunks holding binned surfels
+// and the size of the (tile, chunk) table scan over them.
 struct BinCounts {
-  uint32_t *n_out, *n_rows, *n_band, *n_entries, *n_items, *n_chunks, *n_table;  // n_rows may be null
+  uint32_t *n_out, *n_band, *n_entries, *n_items, *n_chunks, *n_table;
   uint32_t chunk, ntiles;
-  __device__ void set(uint32_t total) const {
+  __device__ void operator()(uint32_t total) const {
     *n_out = total;
-    if (n_rows) *n_rows = 0u;  // null: the spans are computed on another stream
     *n_band = 0u;
     *n_entries = 0u;
     *n_items = 0u;
@@ -373,71 +360,31 @@ struct BinCounts {
   }
 };
 
-struct CompactApply {
-  const uint32_t *zkey;
-  uint32_t *key_out, *val_out;
-  BinCounts bc;
-  using Payload = uint32_t;  // the depth key
-  __device__ Payload fetch(uint32_t i, uint32_t v) const { return v ? zkey[i] : 0u; }
-  __device__ void operator()(uint32_t i, uint32_t prefix, uint32_t v, Payload key) const {
-    if (v) {
-      key_out[prefix] = key;
-      val_out[prefix] = i;
-    }
-  }
-  __device__ void end(uint32_t, uint32_t total) const { bc.set(total); }
-};
-
 // The affiliated eye's surfels in the dominant eye's depth order: a stable filter
 // of that order. For a parallel rig both eyes' keys are identical, so the
 // filtered order is exactly the affiliated (depth, index) order.
 struct ReuseLoad {
-  const uint32_t *uval, *n_union;
+  const uint32_t *order, *n_order;  // the dominant binning's
   uint32_t n_max;
-  const uint32_t *cnt;   // this eye's tile counts
-  const ushort4 *rect;
-  const uint32_t *sat;   // summed-area table of the ROI mask, or null
-  int tiles_x;
+  const uint32_t *bits;             // the selected surfels
   __device__ uint32_t operator()(uint32_t i) const {
-    if (i >= load_n(n_union, n_max)) return 0u;
-    const uint32_t id = uval[i];
-    // the count and the rectangle are loaded together (one memory round trip)
-    const uint32_t c = cnt[id];
-    const ushort4 rc = sat ? rect[id] : make_ushort4(0, 0, 0, 0);
-    if (c == 0u) return 0u;
-    if (!sat) return 1u;
-    return sat_any(sat, tiles_x, rc.y, rc.w, rc.x, rc.z) ? 1u : 0u;
+    if (i >= load_n(n_order, n_max)) return 0u;
+    const uint32_t id = order[i];
+    return (bits[id >> 5] >> (id & 31u)) & 1u;
   }
 };
 
 struct ReuseApply {
-  const uint32_t *uval, *zkey;
-  uint32_t *key_out, *val_out;
+  const uint32_t *order;
+  uint32_t *val_out;
   BinCounts bc;
-  using Payload = uint2;  // surfel id, depth key
-  __device__ Payload fetch(uint32_t i, uint32_t v) const {
-    if (!v) return make_uint2(0u, 0u);
-    const uint32_t id = uval[i];
-    return make_uint2(id, zkey[id]);
+  using Payload = uint32_t;  // surfel id
+  __device__ Payload fetch(uint32_t i, uint32_t v) const { return v ? order[i] : 0u; }
+  __device__ void operator()(uint32_t, uint32_t prefix, uint32_t v, Payload id) const {
+    if (v) val_out[prefix] = id;
   }
-  __device__ void operator()(uint32_t i, uint32_t prefix, uint32_t v, Payload p) const {
-    if (v) {
-      key_out[prefix] = p.y;
-      val_out[prefix] = p.x;
-    }
-  }
-  __device__ void end(uint32_t, uint32_t total) const { bc.set(total); }
+  __device__ void end(uint32_t, uint32_t total) const { bc(total); }
 };
-
-// Keeps the dominant eye's depth order of the union for the affiliated eye.
-__global__ void keep_union_kernel(const uint32_t *__restrict__ src, const uint32_t *__restrict__ n_ptr, uint32_t n_max,
-                                  uint32_t *__restrict__ dst, uint32_t *__restrict__ n_union) {
-  griddep_wait();
-  const uint32_t n = load_n(n_ptr, n_max);
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) dst[i] = src[i];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_union = n;
-}
 
 // ---------------------------------------------------------------- counting sort by tile
 //
@@ -964,75 +911,53 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   if (tile_mask) {  // (the rasterizer-grid mask and) its summed-area table
     launch_k(mask_sat_kernel, 1, 1024, 0, s, const_cast<uint8_t *>(tile_mask), tiles_x, tiles_y, b.mask_sat, roi16,
              (W + kTile - 1) / kTile, (H + kTile - 1) / kTile, roi16 ? tshift : 4, b.mask_clip,
-             roi16 ? b.items16 : nullptr);
+             roi16 ? b.items16 : nullptr, &ctr->n_rows[eye]);
     GS_LAUNCHED(1);
   }
-  // the row spans need only the preprocessed records (and an ROI binning's mask
-  // tables): on a second stream they run beside the compaction and the sort.
-  // Beside a depth sort a small grid leaves those latency-bound kernels their
-  // SMs; beside the filter scan alone (the kept dominant order) the spans are
-  // the longer branch and take a fuller grid
-  const bool side_rows = rows && n > 0;
-  if (side_rows) {
-    const bool reuse = order == kOrderReuse;  // the candidates: the kept dominant order, else every surfel
-    const int cap_g = sm_grid_cap(reuse ? 6 : 2);
+  // 1. the row spans. A full binning's need only the preprocessed records: on a
+  // second stream they run beside the depth order. An ROI binning's select its
+  // surfels for the depth order and come first.
+  const bool side = rows && n > 0 && !tile_mask;
+  const bool sort = order != kOrderReuse;
+  const uint32_t *bits = tile_mask ? b.bits : ws.vis[eye];
+  const auto launch_rows = [&](cudaStream_t st) -> cudaError_t {
+    if (n <= 0) return cudaSuccess;
+    // beside the sort a small grid leaves its latency-bound passes their SMs; with
+    // more surfels the spans are the longer branch, and a third CTA per SM pays
+    // (list start, 2 / 3 per SM: 500k surfels 121 / 125 us, 1.5M 249 / 240, 3M 479 / 444)
+    const int cap_g = sm_grid_cap(side && sort ? (n > (1 << 20) ? 3 : 2) : 6);
     const int grid = cap_g < (n + 255) / 256 ? cap_g : (n + 255) / 256;
-    err = cudaEventRecord(rows->fork, s);
-    if (err == cudaSuccess) err = cudaStreamWaitEvent(rows->stream, rows->fork, 0);
-    if (err == cudaSuccess) err = cudaMemsetAsync(&ctr->n_rows[eye], 0, sizeof(uint32_t), rows->stream);
-    if (err == cudaSuccess)
-      err = launch_k(rows_kernel, grid, 256, 0, rows->stream, reuse ? ws.uval : nullptr,
-                     reuse ? &ctr->n_union : nullptr, (uint32_t)n, ws.rec[eye], ws.rect[eye], ws.cnt[eye], ws.cams,
-                     eye, ws.prim, ws.info[eye], ws.spans[eye], cap, &ctr->n_rows[eye], &ctr->status,
-                     tile_mask ? b.mask_clip : nullptr, tiles_x, tiles_y, tile_mask ? b.mask_sat : nullptr,
-                     reuse ? 0 : 1);
     GS_LAUNCHED(1);
-    if (err == cudaSuccess) err = cudaEventRecord(rows->join, rows->stream);
-    if (err != cudaSuccess) return err;
-  }
+    return launch_k(rows_kernel, grid, 256, 0, st, (uint32_t)n, ws.rec[eye], ws.rect[eye], ws.vis[eye], ws.cams, eye,
+                    ws.prim, ws.info[eye], ws.spans[eye], cap, &ctr->n_rows[eye], &ctr->status,
+                    tile_mask ? b.mask_clip : nullptr, tiles_x, tiles_y, tile_mask ? b.mask_sat : nullptr,
+                    tile_mask ? b.bits : nullptr);
+  };
+  if (!side && (err = launch_rows(s)) != cudaSuccess) return err;
   const uint32_t chunk = kBinWarps * ws.bin_warp_surfels;
-  const BinCounts bc{&ctr->n_vis[eye], side_rows ? nullptr : &ctr->n_rows[eye], &ctr->n_band[eye],
-                     &ctr->n_entries[eye], &ctr->n_items[eye], &ctr->n_chunks[eye], &ctr->n_table[eye], chunk, (uint32_t)ntiles};
-  // 1. compact the binned surfels: (depth bits, surfel id)
-  const uint32_t *sat = tile_mask ? b.mask_sat : nullptr;
-  if (order == kOrderReuse) {  // the dominant order, filtered: already depth-ordered
-    err = scan_launch(ReuseLoad{ws.uval, &ctr->n_union, (uint32_t)n, ws.cnt[eye], ws.rect[eye], sat, tiles_x},
-                      ReuseApply{ws.uval, ws.zkey[eye], b.dkey[0], b.dval[0], bc},
-                      (const uint32_t *)nullptr, (uint32_t)n, b.scan_tiles, b.scan_ticket, &ctr->status, s);
-  } else {
-    err = scan_launch(VisibleLoad{ws.cnt[eye], order == kOrderUnion ? ws.cnt[1 - eye] : nullptr, ws.rect[eye], sat,
-                                  tiles_x},
-                      CompactApply{ws.zkey[eye], b.dkey[0], b.dval[0], bc},
-                      (const uint32_t *)nullptr, (uint32_t)n, b.scan_tiles, b.scan_ticket, &ctr->status, s);
+  const BinCounts bc{&ctr->n_vis[eye], &ctr->n_band[eye], &ctr->n_entries[eye], &ctr->n_items[eye],
+                     &ctr->n_chunks[eye], &ctr->n_table[eye], chunk, (uint32_t)ntiles};
+  // 2. depth order (the low 32 bits of the packed key; stable, so ties keep id
+  // order): the dominant order filtered, or a sort
+  const KeySource src{ws.zkey[eye], bits, order == kOrderUnion ? ws.vis[1 - eye] : nullptr};
+  if (sort && (err = radix_hist(src, (uint32_t)n, rs, bc, s)) != cudaSuccess) return err;
+  if (side) {  // the spans beside the sort's passes: started with the histogram they held the first pass back 20 us
+    if ((err = cudaEventRecord(rows->fork, s)) != cudaSuccess) return err;
+    if ((err = cudaStreamWaitEvent(rows->stream, rows->fork, 0)) != cudaSuccess) return err;
   }
+  err = sort ? radix_passes(src, b.dkey, b.dval, &ctr->n_vis[eye], (uint32_t)n, rs, s)
+             : scan_launch(ReuseLoad{ws.bin[0].dval[0], &ctr->n_vis[0], (uint32_t)n, bits},
+                           ReuseApply{ws.bin[0].dval[0], b.dval[0], bc}, (const uint32_t *)nullptr, (uint32_t)n,
+                           b.scan_tiles, b.scan_ticket, &ctr->status, s);
   if (err != cudaSuccess) return err;
-  // 2. tile ranges of every rectangle row of those surfels (n_rows and n_band
-  // were cleared by the compaction)
-  if (n > 0 && !side_rows) {
-    launch_k(rows_kernel, (n + 255) / 256, 256, 0, s, b.dval[0], &ctr->n_vis[eye], (uint32_t)n, ws.rec[eye],
-                                                ws.rect[eye], ws.cnt[eye], ws.cams, eye, ws.prim, ws.info[eye],
-                                                ws.spans[eye], cap, &ctr->n_rows[eye],
-                                                &ctr->status, tile_mask ? b.mask_clip : nullptr, tiles_x, tiles_y,
-                                                (const uint32_t *)nullptr, order == kOrderReuse ? 0 : 1);
-    GS_LAUNCHED(1);
+  if (side) {
+    if ((err = launch_rows(rows->stream)) != cudaSuccess) return err;
+    if ((err = cudaEventRecord(rows->join, rows->stream)) != cudaSuccess) return err;
+    if ((err = cudaStreamWaitEvent(s, rows->join, 0)) != cudaSuccess) return err;
   }
-  // 3. depth order (the low 32 bits of the packed key; stable, so ties keep id order)
-  int which = 0;
-  if (order != kOrderReuse &&
-      (err = radix_sort(b.dkey, b.dval, &ctr->n_vis[eye], (uint32_t)n, 32, rs, &which, s)) != cudaSuccess)
-    return err;
-  if (order == kOrderUnion && n > 0) {  // kept for the affiliated eye
-    const int cap = sm_grid_cap(8);
-    const int g = (int)((n + 255) / 256 < cap ? (n + 255) / 256 : cap);
-    if ((err = launch_k(keep_union_kernel, g, 256, 0, s, b.dval[which], &ctr->n_vis[eye], (uint32_t)n, ws.uval,
-                        &ctr->n_union)) != cudaSuccess)
-      return err;
-    GS_LAUNCHED(1);
-  }
-  if (side_rows && (err = cudaStreamWaitEvent(s, rows->join, 0)) != cudaSuccess) return err;
-  // 4. per sub-chunk: depth-ordered lists of every tile row's ranges
+  // 3. per sub-chunk: depth-ordered lists of every tile row's ranges
   ListArgs la;
-  la.ids = b.dval[which];
+  la.ids = b.dval[0];
   la.n_vis = &ctr->n_vis[eye];
   la.n_max = (uint32_t)n;
   la.info = ws.info[eye];
@@ -1070,18 +995,18 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   a.cnt_bin = ws.keep_intermediates ? ws.cnt_bin : nullptr;
   if (a.cnt_bin && n > 0 && (err = cudaMemsetAsync(a.cnt_bin, 0, sizeof(uint32_t) * (size_t)n, s)) != cudaSuccess)
     return err;
-  // 5. per-warp counts per (tile, chunk)
+  // 4. per-warp counts per (tile, chunk)
   launch_k(bin_count_kernel, dim3(ws.bin_nch, (unsigned)((tiles_y + kCountRows - 1) / kCountRows)), kBinThreads,
            count_smem_bytes(tiles_x), s, a);
   GS_LAUNCHED(1);
-  // 6. tile-major scan over the chunks that hold binned surfels: where every
+  // 5. tile-major scan over the chunks that hold binned surfels: where every
   // (tile, chunk) run starts, every tile's range and, for a mask, the tile list
   err = scan_launch(BinTableLoad{b.bin_table, &ctr->n_chunks[eye], &ctr->n_vis[eye], ws.bin_nch, chunk},
                     BinOffsetApply{b.bin_offs, &ctr->n_chunks[eye], ws.bin_nch, &ctr->n_inst[eye], &ctr->n_sort[eye],
                                    cap, &ctr->status, b.ranges, ntiles, tile_mask, b.items, &ctr->n_items[eye]},
                     &ctr->n_table[eye], (uint32_t)ntiles * ws.bin_nch, b.scan_tiles, b.scan_ticket, &ctr->status, s);
   if (err != cudaSuccess) return err;
-  // 7. every surfel id to its slot
+  // 6. every surfel id to its slot
   launch_k(bin_place_kernel, dim3(ws.bin_nch, (unsigned)tiles_y), kBinThreads, place_smem_bytes(tiles_x), s, a);
   GS_LAUNCHED(1);
   return cudaGetLastError();

@@ -42,7 +42,7 @@ struct gs_context {
   cudaEvent_t ev_fork, ev_edge, ev_strip;
   cudaEvent_t ev_net;    // learned repair on the second stream: the network is done
   cudaStream_t copy;    // gs_render_stereo_host: the dominant eye's copy to the host
-  cudaStream_t rows;    // the binnings' row spans beside their compaction and sort
+  cudaStream_t rows;    // the full binnings' row spans beside their depth order
   cudaEvent_t ev_rfork, ev_rjoin;
   cudaEvent_t ev_hfork, ev_hjoin;
 };
@@ -73,7 +73,6 @@ bool roi_ok(int gap_thresh, const gs_roi_params *roi);
 bool paths_ok(const gs_context *ctx, const gs_roi_params *roi);
 PoseArgs pose_args(const gs_pose *a, const gs_pose *b, const gs_intrinsics *in, const RasterConfig &rc,
                    const RasterConfig *rc1 = nullptr);
-cudaError_t launch_reset_counters(Counters *c, cudaStream_t s);
 // Copies the optional stereo outputs (class map, ROI rectangles, counts) on ctx->stream.
 cudaError_t copy_optional(gs_context *ctx, const gs_outputs *out, int W, int H);
 int min_tshift(const gs_limits &lim);

@@ -70,7 +70,6 @@ struct Counters {
   uint32_t n_rows[2];    // (surfel, tile row) spans per eye
   uint32_t n_band[2];    // (surfel, band of 4 tile rows) pairs of the last binning per eye
   uint32_t n_entries[2]; // row list entries of the last binning per eye
-  uint32_t n_union;      // surfels in the dominant binning's depth order (both eyes' visible set)
   uint32_t n_items[2];   // rasterizer tiles listed by the last masked binning per eye
   uint32_t prev_range[2];// float bits of the last measured depth range (reused by depth_mode 2)
   uint32_t n_chunks[2];  // binning chunks holding binned surfels, per eye (at least 1)
@@ -95,7 +94,8 @@ struct Record {
 // affiliated eye can be binned and rasterized while the dominant eye's binning
 // and rasterizer run on another stream.
 struct BinScratch {
-  uint32_t *dkey[2], *dval[2];  // depth sort double buffers
+  uint32_t *dkey[2], *dval[2];  // depth sort double buffers; the depth order ends in dval[0]
+  uint32_t *bits;               // an ROI binning's surfels, one bit each
   uint4 *bin_table;             // [tile][chunk] per-warp instance counts (8 x 16 bits)
   struct RowEntry *row_pool;    // (surfel, row range) entries of every warp's lists
   uint2 *row_lists;             // [chunk][row][warp]: first entry, entries
@@ -126,8 +126,8 @@ struct Workspace {
   float4 *bounds[2];
   uint32_t *cnt[2];             // tiles of each surfel's bounding rectangle (0 = culled)
   uint32_t *zkey[2];            // float bits of the centre depth per surfel and eye
+  uint32_t *vis[2];             // one bit per surfel and eye: its rectangle is not empty
   uint32_t *cnt_bin;            // tiles each surfel reaches in the last binning (keep_intermediates)
-  uint32_t *uval;               // depth-ordered union of both eyes' binned surfels (dominant keys)
   uint32_t row_pool_cap[2];     // entries of row_pool, per eye
   uint32_t band_cap[2];         // bound on an eye's (surfel, band of 4 tile rows) pairs
   BinScratch bin[2];            // per eye
@@ -190,7 +190,8 @@ size_t workspace_bytes(const gs_limits &lim);
 bool carve_workspace(const gs_limits &lim, void *base, size_t bytes, Workspace *ws);
 
 // ---- launches (each returns the launch error) ----
-cudaError_t launch_setup_cams(const PoseArgs &pa, CamBlock *cams, cudaStream_t s);
+cudaError_t launch_setup_cams(const PoseArgs &pa, CamBlock *cams, Counters *ctr, cudaStream_t s);
+constexpr int kSetupThreads = 32;
 // Address of the set-up kernel (its graph node carries the per-frame poses).
 const void *setup_cams_kernel_ptr();
 cudaError_t launch_preprocess(const gs_scene &sc, Workspace &ws, int neyes, int W, int H,
@@ -199,9 +200,9 @@ cudaError_t launch_preprocess(const gs_scene &sc, Workspace &ws, int neyes, int 
 // sorted per-tile instance lists and their ranges. Depth order:
 //   kOrderOwn     sort this eye's binned surfels by their own keys;
 //   kOrderUnion   (dominant eye of a parallel two-eye call) sort every surfel
-//                 either eye bins by the dominant keys and keep that order in
-//                 ws.uval;
-//   kOrderReuse   (affiliated eye after kOrderUnion) filter the kept order: for
+//                 either eye bins by the dominant keys;
+//   kOrderReuse   (affiliated eye after kOrderUnion) filter that order, which the
+//                 dominant eye's scratch still holds: for
 //                 a parallel rig both eyes' depth keys are identical, so the
 //                 filtered order is the affiliated (depth, index) order.
 enum BinOrder { kOrderOwn = 0, kOrderUnion = 1, kOrderReuse = 2 };
@@ -209,9 +210,8 @@ enum BinOrder { kOrderOwn = 0, kOrderUnion = 1, kOrderReuse = 2 };
 // ROI mask on the 16-pixel grid from which the binning derives its own mask on
 // the rasterizer grid into tile_mask (then ws.bin[eye].rmask); null when
 // tile_mask is given directly (or no mask).
-// rows (optional): a second stream and two events on which the row spans are
-// computed beside the compaction and the depth sort (forked after the mask
-// tables, joined before the band lists); null: on s, after the compaction.
+// rows (optional): a second stream and two events on which a full binning's row
+// spans are computed beside its depth order (joined before the row lists).
 struct SideRows {
   cudaStream_t stream;
   cudaEvent_t fork, join;

@@ -9,58 +9,76 @@
 
 namespace gs {
 
-// ---------------------------------------------------------------- FP64 set-up
+// ---------------------------------------------------------------- set-up
 //
 // The only double-precision work on the GPU: inverting the camera-to-world
 // poses (world -> camera) and composing the relative pose between the eyes,
 // X_aff = R_aff^T R_dom X_dom + R_aff^T (t_dom - t_aff) (Eq. 4 followed by Eq. 5).
-__global__ void setup_cams_kernel(PoseArgs pa, CamBlock *cams) {
+// Every frame starts with this kernel, and FP64 is slow here: lane 3 e + i takes
+// row i of eye e's camera, lanes 6-8 a row of the relative pose each (one thread
+// for all took 5 us), and another lane resets the frame's counters.
+__global__ void __launch_bounds__(kSetupThreads) setup_cams_kernel(PoseArgs pa, CamBlock *cams, Counters *ctr) {
   griddep_wait();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  CamBlock cb;
-  for (int e = 0; e < 2; ++e) {
-    const int src = e < pa.neyes ? e : 0;
-    const double *R = pa.R[src], *t = pa.t[src];
-    EyeCam &c = cb.eye[e];
-    for (int i = 0; i < 3; ++i) {
+  const int l = threadIdx.x;
+  if (l < 6) {
+    const int e = l / 3, i = l % 3;
+    const auto row = [&](int src) {
       double ti = 0.0;
-      for (int j = 0; j < 3; ++j) {
-        c.R[i * 3 + j] = (float)R[j * 3 + i];  // transpose
-        ti -= R[j * 3 + i] * t[j];
-      }
-      c.t[i] = (float)ti;
-      c.centre[i] = (float)t[i];
+      for (int j = 0; j < 3; ++j) ti -= pa.R[src][j * 3 + i] * pa.t[src][j];
+      return (float)ti;
+    };
+    const int src = e < pa.neyes ? e : 0;
+    EyeCam &c = cams->eye[e];
+    for (int j = 0; j < 3; ++j) c.R[i * 3 + j] = (float)pa.R[src][j * 3 + i];  // transpose
+    // A parallel rig (equal orientation, baseline in the image plane, Sec. 4.2):
+    // both cameras measure the same depth, z_aff = z_dom in exact arithmetic. The
+    // two offsets differ only by FP64 rounding of R^T R = I, so the affiliated eye
+    // takes the dominant one and both eyes' depth keys are bit-identical.
+    c.t[i] = row(pa.parallel && i == 2 ? 0 : src);
+    c.centre[i] = (float)pa.t[src][i];
+  } else if (l < 9) {
+    const int i = l - 6, a = pa.neyes > 1 ? 1 : 0;
+    const double *Rd = pa.R[0], *td = pa.t[0], *Ra = pa.R[a], *ta = pa.t[a];
+    double tr = 0.0;
+    for (int j = 0; j < 3; ++j) {
+      double r = 0.0;
+      for (int k = 0; k < 3; ++k) r += Ra[k * 3 + i] * Rd[k * 3 + j];
+      cams->Rrel[i * 3 + j] = (float)r;
+      tr += Ra[j * 3 + i] * (td[j] - ta[j]);
     }
+    cams->trel[i] = (float)tr;
+  } else if (l < 11) {
+    const int e = l - 9;
+    EyeCam &c = cams->eye[e];
     c.fx = (float)pa.fx; c.fy = (float)pa.fy; c.cx = (float)pa.cx; c.cy = (float)pa.cy;
     c.W = pa.W; c.H = pa.H;
     c.tshift = e == 0 ? pa.tshift : pa.tshift1;
     c.tiles_x = (pa.W + (1 << c.tshift) - 1) >> c.tshift;
     c.tiles_y = (pa.H + (1 << c.tshift) - 1) >> c.tshift;
-  }
-  // A parallel rig (equal orientation, baseline in the image plane, Sec. 4.2):
-  // both cameras measure the same depth, z_aff = z_dom in exact arithmetic. The
-  // two offsets differ only by FP64 rounding of R^T R = I, so the affiliated eye
-  // takes the dominant one and both eyes' depth keys are bit-identical.
-  if (pa.parallel) cb.eye[1].t[2] = cb.eye[0].t[2];
-  const int a = pa.neyes > 1 ? 1 : 0;
-  const double *Rd = pa.R[0], *td = pa.t[0], *Ra = pa.R[a], *ta = pa.t[a];
-  for (int i = 0; i < 3; ++i) {
-    double tr = 0.0;
-    for (int j = 0; j < 3; ++j) {
-      double r = 0.0;
-      for (int k = 0; k < 3; ++k) r += Ra[k * 3 + i] * Rd[k * 3 + j];
-      cb.Rrel[i * 3 + j] = (float)r;
-      tr += Ra[j * 3 + i] * (td[j] - ta[j]);
+  } else if (l < 13) {
+    const int e = l - 11;
+    ctr->n_vis[e] = 0;
+    ctr->n_inst[e] = 0;
+    ctr->n_sort[e] = 0;
+    ctr->n_rows[e] = 0;
+    ctr->n_band[e] = 0;
+    ctr->n_entries[e] = 0;
+    ctr->n_items[e] = 0;
+    ctr->pairs[e] = 0ull;
+    ctr->contrib[e] = 0ull;
+    if (e == 0) {
+      ctr->dmin_bits = 0x7f800000u;
+      ctr->dmax_bits = 0u;
+      ctr->n_rects = 0;
+      ctr->n_centre = 0;
     }
-    cb.trel[i] = (float)tr;
   }
-  *cams = cb;
 }
 
 const void *setup_cams_kernel_ptr() { return (const void *)setup_cams_kernel; }
 
-cudaError_t launch_setup_cams(const PoseArgs &pa, CamBlock *cams, cudaStream_t s) {
-  launch_k(setup_cams_kernel, 1, 32, 0, s, pa, cams);
+cudaError_t launch_setup_cams(const PoseArgs &pa, CamBlock *cams, Counters *ctr, cudaStream_t s) {
+  launch_k(setup_cams_kernel, 1, kSetupThreads, 0, s, pa, cams, ctr);
   GS_LAUNCHED(1);
   return cudaGetLastError();
 }
@@ -249,6 +267,9 @@ __global__ void __launch_bounds__(256) preprocess_kernel(gs_scene sc, const CamB
       count = 0;
       rect = make_ushort4(0, 0, 0, 0);
     }
+    // (the lanes past the last surfel have left the kernel)
+    const uint32_t seen = __ballot_sync(0xffffffffu, count > 0u);
+    if ((threadIdx.x & 31) == 0) ws.vis[e][i >> 5] = seen;
     ws.cnt[e][i] = count;
     ws.rect[e][i] = rect;
     ws.zkey[e][i] = __float_as_uint(pc[2]);
@@ -345,6 +366,9 @@ __global__ void __launch_bounds__(256) preprocess_ellipsoid_kernel(gs_scene sc, 
       count = 0;
       rect = make_ushort4(0, 0, 0, 0);
     }
+    // (the lanes past the last surfel have left the kernel)
+    const uint32_t seen = __ballot_sync(0xffffffffu, count > 0u);
+    if ((threadIdx.x & 31) == 0) ws.vis[e][i >> 5] = seen;
     ws.cnt[e][i] = count;
     ws.rect[e][i] = rect;
     ws.zkey[e][i] = __float_as_uint(pc[2]);

@@ -1,9 +1,14 @@
 // Stable LSD radix sort of (uint32 key, uint32 value) pairs, 8 bits per pass,
-// with a device-resident element count ("one sweep" per pass).
+// with a device-resident element count ("one sweep" per pass). The pairs are the
+// selected indices i < n of a key array, with their keys: the histogram and the
+// first pass read the array through the selection (one bit per index), so the
+// selected pairs are never compacted first (that scan took 20 of the 87 us of a
+// sort of 470k of 500k surfels, 50 of 226 at 1.9M of 3M).
 //
 //   1. One histogram kernel counts every pass's digits over all keys at once
 //      (the digit counts of a pass do not depend on the order the earlier
-//      passes leave); the last CTA out turns them into each pass's digit bases.
+//      passes leave); the last CTA out turns them into each pass's digit bases
+//      and hands the number of pairs to the caller's functor.
 //   2. Per pass, one kernel: a CTA takes the next tile of 2048 pairs from a
 //      device counter, ranks its pairs stably (per warp with bit ballots, then
 //      across warps), publishes its per-digit counts, and finds every digit's
@@ -46,23 +51,48 @@ inline int radix_hist_grid(uint32_t n_max) {
   return (int)(tiles < 1 ? 1 : (tiles > cap ? cap : tiles));
 }
 
-// Digit counts of all passes; the last CTA out writes the bases and clears the
-// counts and its ticket.
-static __global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(const uint32_t *__restrict__ keys,
-                                                                     const uint32_t *n_ptr, uint32_t n_max,
-                                                                     int npass, RadixScratch sc) {
+// The sorted pairs: indices i < n whose bit is set in `bits` (or, if given, in
+// `bits_or`), with key[i].
+struct KeySource {
+  const uint32_t *key, *bits, *bits_or;
+  __device__ __forceinline__ bool has(uint32_t i) const {
+    uint32_t w = bits[i >> 5];
+    if (bits_or) w |= bits_or[i >> 5];
+    return (w >> (i & 31u)) & 1u;
+  }
+};
+
+// Digit counts of all passes; the last CTA out writes the bases, hands the pairs'
+// number to done(n) and clears the counts and its ticket.
+template <class Done>
+static __global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(KeySource src, uint32_t n, RadixScratch sc,
+                                                                     Done done) {
   griddep_wait();
   __shared__ uint32_t h[kRsPasses][256];
   __shared__ uint32_t s_last, s_scan[32];
   for (int i = threadIdx.x; i < kRsPasses * 256; i += kRsThreads) (&h[0][0])[i] = 0u;
   __syncthreads();
-  const uint32_t n = load_n(n_ptr, n_max);
-  for (uint32_t i = blockIdx.x * kRsThreads + threadIdx.x; i < n; i += gridDim.x * kRsThreads) {
-    const uint32_t k = keys[i];
-    for (int p = 0; p < npass; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 255u], 1u);
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t i0 = (blockIdx.x * kRsThreads + threadIdx.x) & ~31u; i0 < n; i0 += gridDim.x * kRsThreads) {
+    const uint32_t i = i0 + lane;  // warp-uniform loop
+    const bool ok = i < n && src.has(i);
+    const uint32_t k = ok ? src.key[i] : 0u;
+    if (ok) {
+#pragma unroll
+      for (int p = 0; p < kRsPasses - 1; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 255u], 1u);
+    }
+    // the top digit of depths within a factor of four is one of two values: a
+    // vote per value in place of 32 atomics on one address
+    uint32_t todo = __ballot_sync(0xffffffffu, ok);
+    while (todo) {
+      const uint32_t d = __shfl_sync(0xffffffffu, k >> 24, __ffs((int)todo) - 1);
+      const uint32_t same = __ballot_sync(0xffffffffu, ok && (k >> 24) == d);
+      if (lane == 0) atomicAdd(&h[kRsPasses - 1][d], (uint32_t)__popc(same));
+      todo &= ~same;
+    }
   }
   __syncthreads();
-  for (int p = 0; p < npass; ++p) {
+  for (int p = 0; p < kRsPasses; ++p) {
     const uint32_t v = h[p][threadIdx.x];
     if (v) atomicAdd(&sc.hist[p * 256 + threadIdx.x], v);
   }
@@ -78,14 +108,18 @@ static __global__ void __launch_bounds__(kRsThreads) rs_hist_kernel(const uint32
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int p = 0; p < npass; ++p) {
+  uint32_t total = 0;
+  for (int p = 0; p < kRsPasses; ++p) {
     const uint32_t v = __ldcg(&sc.hist[p * 256 + threadIdx.x]);
     uint32_t ex;
-    block_exclusive_scan<kRsThreads>(v, &ex, s_scan);
+    total = block_exclusive_scan<kRsThreads>(v, &ex, s_scan);
     sc.base[p * 256 + threadIdx.x] = ex;
     sc.hist[p * 256 + threadIdx.x] = 0u;
   }
-  if (threadIdx.x == 0) sc.ctl[3] = 0u;
+  if (threadIdx.x == 0) {
+    sc.ctl[3] = 0u;
+    done(total);
+  }
 }
 
 // Sum of digit d's counts over tiles [0, t) (t > 0) by decoupled look-back.
@@ -119,7 +153,9 @@ __device__ __forceinline__ uint32_t rs_lookback(const unsigned long long *status
   return prefix;
 }
 
-static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(const uint32_t *__restrict__ kin,
+// FIRST: the pairs come from src (n_max indices), else from kin / vin (*n_ptr pairs).
+template <bool FIRST>
+static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(KeySource src, const uint32_t *__restrict__ kin,
                                                                       const uint32_t *__restrict__ vin,
                                                                       uint32_t *__restrict__ kout,
                                                                       uint32_t *__restrict__ vout,
@@ -139,23 +175,30 @@ static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(const uint3
   __syncthreads();
   const uint32_t t = s_tile;
   const uint32_t epoch = (*(volatile uint32_t *)(sc.ctl + 2)) & 0x3fffffffu;
-  const uint32_t n = load_n(n_ptr, n_max);
+  const uint32_t n = FIRST ? n_max : load_n(n_ptr, n_max);
   const uint32_t base = t * (uint32_t)kRsTile;
   if (base < n) {
     for (int i = tid; i < NW * 256; i += kRsThreads) (&s_warp[0][0])[i] = 0;
     __syncthreads();
     // warp w owns pairs [w * 32 * kRsItems, (w + 1) * 32 * kRsItems) of the tile
     uint32_t k[kRsItems], r[kRsItems], v[kRsItems];
+    uint32_t have = 0;  // bit j: item j is a pair
 #pragma unroll
     for (int j = 0; j < kRsItems; ++j) {  // values loaded with the keys: no second wait
       const uint32_t i = base + (uint32_t)(wid * 32 * kRsItems + j * 32 + lane);
-      k[j] = i < n ? kin[i] : 0u;
-      v[j] = i < n ? vin[i] : 0u;
+      if (FIRST) {
+        k[j] = i < n ? src.key[i] : 0u;
+        v[j] = i;
+        if (i < n && src.has(i)) have |= 1u << j;
+      } else {
+        k[j] = i < n ? kin[i] : 0u;
+        v[j] = i < n ? vin[i] : 0u;
+        if (i < n) have |= 1u << j;
+      }
     }
 #pragma unroll
     for (int j = 0; j < kRsItems; ++j) {
-      const uint32_t i = base + (uint32_t)(wid * 32 * kRsItems + j * 32 + lane);
-      const bool ok = i < n;
+      const bool ok = (have >> j) & 1u;
       const uint32_t d = (k[j] >> shift) & 255u;
       // lanes holding the same digit: intersect one ballot per digit bit
       uint32_t peers = __ballot_sync(0xffffffffu, ok);
@@ -192,16 +235,13 @@ static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(const uint3
       lb_store(my, epoch, kLbIncl, prefix + cnt);
     }
     s_global[tid] = __ldg(&sc.base[pass * 256 + tid]) + prefix;
-    {
-      uint32_t ex;
-      block_exclusive_scan<kRsThreads>(cnt, &ex, s_scan);
-      s_local_base[tid] = ex;
-    }
+    uint32_t ex;
+    const uint32_t tn = block_exclusive_scan<kRsThreads>(cnt, &ex, s_scan);  // the tile's pairs
+    s_local_base[tid] = ex;
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kRsItems; ++j) {
-      const uint32_t i = base + (uint32_t)(wid * 32 * kRsItems + j * 32 + lane);
-      if (i < n) {
+      if ((have >> j) & 1u) {
         const uint32_t d = (k[j] >> shift) & 255u;
         const uint32_t pos = s_local_base[d] + s_warp[wid][d] + r[j];
         s_keys[pos] = k[j];
@@ -209,7 +249,6 @@ static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(const uint3
       }
     }
     __syncthreads();
-    const uint32_t tn = min((uint32_t)kRsTile, n - base);
     for (uint32_t i = tid; i < tn; i += kRsThreads) {
       const uint32_t key = s_keys[i];
       const uint32_t d = (key >> shift) & 255u;
@@ -230,22 +269,26 @@ static __global__ void __launch_bounds__(kRsThreads) rs_sweep_kernel(const uint3
   }
 }
 
-// Sorts on bits [0, bits) (bits <= 32); the result lands in buffer index *which.
-inline cudaError_t radix_sort(uint32_t *const keys[2], uint32_t *const vals[2], const uint32_t *n_ptr, uint32_t n_max,
-                              int bits, const RadixScratch &sc, int *which, cudaStream_t s) {
-  const int npass = (bits + 7) / 8;
-  const int tiles = (int)((n_max + kRsTile - 1) / kRsTile);
-  launch_k(rs_hist_kernel, radix_hist_grid(n_max), kRsThreads, 0, s, (const uint32_t *)keys[0], n_ptr, n_max, npass,
-           sc);
+// Sorts the pairs of src over all 32 key bits into keys[0] / vals[0]: the histogram,
+// then the passes. The pairs' number is at n_ptr once the histogram's done(n) has
+// stored it there.
+template <class Done>
+cudaError_t radix_hist(const KeySource &src, uint32_t n_max, const RadixScratch &sc, Done done, cudaStream_t s) {
   GS_LAUNCHED(1);
-  int cur = 0;
-  for (int p = 0; p < npass; ++p) {
-    launch_k(rs_sweep_kernel, tiles < 1 ? 1 : tiles, kRsThreads, 0, s, (const uint32_t *)keys[cur],
-             (const uint32_t *)vals[cur], keys[cur ^ 1], vals[cur ^ 1], n_ptr, n_max, p, sc);
-    GS_LAUNCHED(1);
-    cur ^= 1;
-  }
-  *which = cur;
+  return launch_k(rs_hist_kernel<Done>, radix_hist_grid(n_max), kRsThreads, 0, s, src, n_max, sc, done);
+}
+
+inline cudaError_t radix_passes(const KeySource &src, uint32_t *const keys[2], uint32_t *const vals[2],
+                                const uint32_t *n_ptr, uint32_t n_max, const RadixScratch &sc, cudaStream_t s) {
+  const int tiles = (int)((n_max + kRsTile - 1) / kRsTile);
+  const int grid = tiles < 1 ? 1 : tiles;
+  launch_k(rs_sweep_kernel<true>, grid, kRsThreads, 0, s, src, (const uint32_t *)nullptr, (const uint32_t *)nullptr,
+           keys[1], vals[1], n_ptr, n_max, 0, sc);
+  static_assert(kRsPasses % 2 == 0, "the last pass writes buffer 0");
+  for (int p = 1; p < kRsPasses; ++p)
+    launch_k(rs_sweep_kernel<false>, grid, kRsThreads, 0, s, src, (const uint32_t *)keys[p & 1],
+             (const uint32_t *)vals[p & 1], keys[(p & 1) ^ 1], vals[(p & 1) ^ 1], n_ptr, n_max, p, sc);
+  GS_LAUNCHED(kRsPasses);
   return cudaGetLastError();
 }
 
