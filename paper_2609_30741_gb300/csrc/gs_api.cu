@@ -9,6 +9,7 @@
 #include "gs_context.cuh"
 #include "gs_launch.cuh"
 #include "gs_sort.cuh"
+#include "gs_warp.cuh"
 
 namespace gs {
 
@@ -133,6 +134,7 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   ws.rp_list = c.take<uint32_t>(tiles);
   ws.rp_nlist = c.take<uint32_t>(1);
   ws.ssim_part = c.take<double>(ssim_partials(lim.max_width, lim.max_height));
+  ws.ssim_ticket = c.take<uint32_t>(1);
   ws.strips = c.take<int32_t>(16);
   ws.drange = c.take<float>(2);
   ws.widths = c.take<int32_t>(4);
@@ -267,6 +269,11 @@ PoseArgs pose_args(const gs_pose *a, const gs_pose *b, const gs_intrinsics *in, 
   }
   pa.fx = in->fx; pa.fy = in->fy; pa.cx = in->cx; pa.cy = in->cy;
   pa.W = in->width; pa.H = in->height;
+  if (b) {
+    double Rrel[9], trel[3];
+    relative_pose(a->R, a->t, b->R, b->t, Rrel, trel);
+    pa.rows = rows_kept(Rrel, trel, in->fx, in->fy, in->cx, in->cy, in->width, in->height) ? 1 : 0;
+  }
   return pa;
 }
 
@@ -388,6 +395,7 @@ gs_status gs_context_create(gs_context **out, const gs_limits *lim, void *worksp
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.bin[k].rs_ctl, 0, sizeof(uint32_t) * 4, ctx->stream);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ctr, 0, sizeof(Counters), ctx->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ws.ssim_ticket, 0, sizeof(uint32_t), ctx->stream);
   if (e != cudaSuccess) {
     delete ctx;
     return cuda_fail(e);
@@ -787,6 +795,7 @@ static gs_status stereo_impl(gs_context *ctx, const gs_scene *scene, const gs_po
   kb.add(r);
   kb.add(*out);
   kb.add(pa.parallel);  // selects the depth-order path of the affiliated eye
+  kb.add(pa.rows);      // and the warp's
   kb.add(rc1);
   kb.add(hc ? hc->dom : nullptr);  // host copies are nodes of the captured graph
   kb.add(hc ? hc->aff : nullptr);
@@ -835,10 +844,10 @@ static gs_status stereo_impl(gs_context *ctx, const gs_scene *scene, const gs_po
       if (e != cudaSuccess) return cuda_fail(e);
     }
     // Stage 1: dominant eye, RGB + depth proxy (+ the per-frame depth range)
-    // without a reused depth range the dominant eye's rasterizer also clears the
-    // warp buffer (the two eyes share the image size)
+    // the dominant eye's rasterizer also clears the warp buffer (the two eyes share
+    // the image size), unless the range is reused or the warp writes it row by row
     st = render_eye_full(ctx, scene, 0, W, H, black, out->rgb_dom, out->depth_dom, out->trans_dom, true, 2,
-                         p.parallel ? kOrderUnion : kOrderOwn, reuse ? nullptr : ws.warpbuf);
+                         p.parallel ? kOrderUnion : kOrderOwn, reuse || p.rows ? nullptr : ws.warpbuf);
     if (st != GS_OK) return st;
     if (hc) {  // the dominant eye is final: copy it out beside Stages 2-4
       if ((e = cudaEventRecord(ctx->ev_hfork, ctx->stream)) == cudaSuccess)
@@ -851,12 +860,12 @@ static gs_status stereo_impl(gs_context *ctx, const gs_scene *scene, const gs_po
     }
     // Stages 2-3: warp, edge ROIs, gaps
     if (reuse) {
-      e = launch_warp(ws, W, H, out->depth_dom, out->trans_dom, ctx->stream);
+      e = launch_warp(ws, W, H, out->depth_dom, out->trans_dom, p.rows != 0, ctx->stream);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->stream, ctx->ev_edge, 0);
       if (e == cudaSuccess) e = launch_classify(ws, W, H, gap_thresh, r, out->rgb_dom, out->rgb_aff, ctx->stream);
     } else {
       e = launch_warp_classify(ws, W, H, gap_thresh, r, out->rgb_dom, out->depth_dom, out->trans_dom, out->rgb_aff,
-                               ctx->stream, true);
+                               ctx->stream, p.rows != 0, true);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     if (r.repair_mode != 0) {  // the repair network's inputs, kept for gs_repair_features
@@ -989,7 +998,8 @@ gs_status gs_ssim(gs_context *ctx, const float *img, const float *ref, int width
   if (!ctx || !img || !ref || !ssim || width <= 0 || height <= 0 || width > ctx->lim.max_width ||
       height > ctx->lim.max_height || channels < 1 || channels > 3)
     return GS_ERR_BAD_ARG;
-  return cuda_status(launch_ssim(img, ref, width, height, channels, ctx->ws.ssim_part, ssim, ctx->stream));
+  return cuda_status(launch_ssim(img, ref, width, height, channels, ctx->ws.ssim_part, ctx->ws.ssim_ticket, ssim,
+                                 ctx->stream));
 }
 
 gs_status gs_centre_rois(gs_context *ctx, const uint8_t *cls, int width, int height, int margin, int32_t *rects,

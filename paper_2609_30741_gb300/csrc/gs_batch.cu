@@ -166,7 +166,7 @@ static gs_status enqueue_batch(gs_batch *b, const gs_frame *frames, int n, const
       continue;
     }
     BTRY(launch_warp_classify(ctx->ws, g[f].W, g[f].H, gap_thresh, *roi, o.rgb_dom, o.depth_dom, o.trans_dom,
-                              o.rgb_aff, s));
+                              o.rgb_aff, s, g[f].pa.rows != 0));
     if (roi->repair_mode != 0) BTRY(repair_features(ctx->ws, g[f].W, g[f].H, o.rgb_aff, ctx->ws.rp_feat, s));
     if (roi->enable_center) BTRY(launch_centre_rois(ctx->ws, g[f].W, g[f].H, roi->margin, s));
     if (roi->repair_mode == 1 || roi->repair_mode == 2)
@@ -352,6 +352,7 @@ static void key_frames(KeyBuilder &kb, gs_batch *b, int kind, const gs_frame *fr
     kb.add(frames[f].intr.height);
     kb.add(frames[f].out);
     kb.add(g[f].pa.parallel);
+    kb.add(g[f].pa.rows);
   }
 }
 

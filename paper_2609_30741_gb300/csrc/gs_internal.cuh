@@ -56,6 +56,7 @@ struct PoseArgs {
   int W, H;
   int neyes;
   int parallel;  // the eyes share orientation and the baseline lies in the image plane
+  int rows;      // every warped sample keeps its image row (rows_kept)
   int tshift;    // rasterizer tile edge = 1 << tshift pixels (the dominant eye)
   int tshift1;   // the affiliated eye's (its ROI re-render may use another tile edge)
 };
@@ -161,6 +162,7 @@ struct Workspace {
   uint8_t *rp_skip;             // [16-pixel tiles] the network's fill was taken
   uint32_t *rp_list, *rp_nlist; // listed tiles and their number
   double *ssim_part;            // per-(tile, channel) SSIM sums
+  uint32_t *ssim_ticket;        // CTAs done (zero between launches)
   // limits
   int max_surfels, max_w, max_h, max_rects, max_tiles;  // max_tiles: rasterizer tiles at min_tshift
   int min_tshift;               // smallest rasterizer tile edge the buffers hold (log2)
@@ -331,17 +333,18 @@ cudaError_t launch_lpt_order(RasterFrame &f, uint32_t *buf, cudaStream_t s);
 RasterFrame raster_frame(const Workspace &ws, int eye, int W, int H, int tshift, const uint8_t *mask, float3 bg,
                          float *rgb, float *depth, float *trans, uint8_t *cls, bool stats);
 // Mean SSIM of a [C][H][W] image against a reference (11 x 11 Gaussian window,
-// zero padding) into *out (device); part: ssim_partials() doubles.
+// zero padding) into *out (device); part: ssim_partials() doubles; *ticket is zero
+// between launches.
 size_t ssim_partials(int max_w, int max_h);
-cudaError_t launch_ssim(const float *a, const float *b, int W, int H, int C, double *part, float *out,
+cudaError_t launch_ssim(const float *a, const float *b, int W, int H, int C, double *part, uint32_t *ticket, float *out,
                         cudaStream_t s);
-// The stages of launch_warp_classify one by one: the warp (clears the warp
-// buffer and the ROI mask first), the edge ROI (into `mask`: ORed into the
+// The stages of launch_warp_classify one by one: the warp (clears the ROI mask and
+// writes the whole warp buffer; rows: PoseArgs::rows), the edge ROI (into `mask`: ORed into the
 // cleared ROI mask, or every tile assigned when `assign`), and the
 // classification (which also keeps this frame's measured depth range for the
 // next frame's depth_mode 2).
 cudaError_t launch_warp(const Workspace &ws, int W, int H, const float *depth_dom, const float *trans_dom,
-                        cudaStream_t s);
+                        bool rows, cudaStream_t s);
 // Value of an empty warp-buffer entry (no source pixel landed there).
 constexpr unsigned long long kNoSample = ~0ull;
 cudaError_t launch_edge_roi(const Workspace &ws, const gs_roi_params &roi, uint8_t *mask, bool assign,
@@ -353,12 +356,13 @@ cudaError_t launch_strip_composite(const Workspace &ws, int W, int H, const floa
                                    cudaStream_t s);
 cudaError_t launch_mask_minus(uint8_t *mask, const uint8_t *minus, int n, cudaStream_t s);
 // Warp, edge ROIs, hole classification and gap filling (writes rgb_aff and cls).
-// cleared = true: the dominant eye's rasterizer has cleared the warp buffer
-// (RasterFrame::winit), and the edge ROI assigns every tile of the ROI mask
-// instead of adding its strips to a cleared mask.
+// rows: PoseArgs::rows. cleared = true (without rows): the dominant eye's
+// rasterizer has cleared the warp buffer (RasterFrame::winit). In both cases the
+// edge ROI assigns every tile of the ROI mask; else it adds its strips to a mask
+// that is cleared with the buffer.
 cudaError_t launch_warp_classify(const Workspace &ws, int W, int H, int gap_thresh, const gs_roi_params &roi,
                                  const float *rgb_dom, const float *depth_dom, const float *trans_dom,
-                                 float *rgb_aff, cudaStream_t s, bool cleared = false);
+                                 float *rgb_aff, cudaStream_t s, bool rows, bool cleared = false);
 // Connected centre holes -> ROI rectangles -> tile mask.
 cudaError_t launch_centre_rois(const Workspace &ws, int W, int H, int margin, cudaStream_t s);
 
