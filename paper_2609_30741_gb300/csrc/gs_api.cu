@@ -67,9 +67,15 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   const size_t table = tiles * ws.bin_nch;
   ws.cnt_bin = c.take<uint32_t>(lim.keep_intermediates ? N : 1);
   // the row-list entries are the spans, but for an ROI binning's rows without a
-  // masked tile, and one more for each of the few spans with two ranges
+  // masked tile, and one more for each of the few spans with two ranges: an eighth
+  // more entries than spans hold them (9 B per span). 12 B for each of the first 8
+  // spans per surfel cover that; for capacities far beyond, both eyes' pools get
+  // what the larger one still needs.
+  const size_t few = 8 * N, most = Ie[0] > Ie[1] ? Ie[0] : Ie[1];
+  const size_t pool_more = 9 * most > 12 * few ? 9 * most - 12 * few : 0;
   for (int e = 0; e < 2; ++e) {
-    ws.row_pool_cap[e] = (uint32_t)(Ie[e] + Ie[e] / 8 + 1024);
+    const size_t bytes = 12 * (Ie[e] < few ? Ie[e] : few) + pool_more;
+    ws.row_pool_cap[e] = (uint32_t)(bytes / kRowEntryBytes + 1024);
     ws.band_cap[e] = (uint32_t)(Ie[e] < 8 * N ? Ie[e] + 1024 : 8 * N + 1024);
   }
   const size_t rs_words = radix_status_words(N);
