@@ -97,15 +97,23 @@ static_assert(kWPackTBytes == 82944, "packed transposed weight image size");
 __host__ __device__ constexpr int vrows(int l) { return kGW - 2 * (l + 1); }            // layer l's output edge
 __host__ __device__ constexpr int kchunks(int l) { return (vrows(l) * kGW + 15) / 16; }  // weight-gradient K = 16 steps
 constexpr int kBwdThreads = 256;
-constexpr int kBwdTmemCols = 512;   // 9 taps x 32 (weight gradient) + 6 M tiles x 32 (input gradient)
-constexpr int kBufT = (kchunks(0) + 2) * 1024;  // dY^T, plus the reach of the padded A rows
-constexpr int kBwdParts = 32 * 9 * 32 + 32;     // largest layer: weight and bias gradients
-static_assert(9 * 32 + kMaxMT * 32 <= kBwdTmemCols, "tensor memory of the backward");
-static_assert(kchunks(0) * 16 + 2 * kGW + 2 <= kNPos && kMaxMT * 128 + 2 * kGW + 2 <= kNPos,
-              "backward operand reach");
+constexpr int kBwdTmemCols = 512;   // 3 tap rows x 32 (weight gradient) + 6 M tiles x 32 (input gradient)
+// dY in shared memory: planes [horizontal tap s][c_out group] of kDPlane positions,
+// dY at position q stored kDPad + s + q into its plane, zero elsewhere
+constexpr int kDPlane = 800;
+constexpr int kDRegs = 3;  // positions of a plane a thread stages
+static_assert(3 * 32 + kMaxMT * 32 <= kBwdTmemCols, "tensor memory of the backward");
+static_assert(kchunks(0) * 16 + 2 * kGW + 2 <= kNPos, "weight gradient: reach of x");
+static_assert(kDPad + 2 + kchunks(0) * 16 <= kDPlane && kchunks(0) * 16 <= kDRegs * kBwdThreads, "a plane holds dY");
+// the input gradient reads dY at positions < kDPad + vin * 28 of a plane, its unused rows a little of the next;
+// 16 groups of M = 128 rows read 4 planes past the 12
+static_assert(vrows(0) * kGW + kDPad <= kDPlane && kMaxMT * 128 + kDPad <= kDPlane + kDPad, "input gradient: reach of dY");
+constexpr size_t kBufD = 12 * (size_t)kDPlane * 16;
+static_assert(4 * (size_t)kDPlane * 16 <= 4 * (size_t)kNPos * 16, "reach of the unused rows");
 __host__ __device__ constexpr size_t bwd_smem() {
-  return 128 + 2 * (size_t)(4 * kNPos * 16) + kBufT + wbytesT(1) + (8 * 32 + 32) * 4 + 2 * 8 + 16;
+  return 128 + kBufD + 4 * (size_t)kNPos * 16 + wbytesT(1) + (8 * 32 + 32) * 4 + (kMaxMT + 1) * 8 + 16;
 }
+static_assert(bwd_smem() <= 227 * 1024, "shared memory of the backward");
 static_assert(kMaxMT * 128 + 2 * kGW + 2 <= kNPos, "activation buffer reach");
 // shared memory of the network kernel: two activation buffers, the weight image,
 // bias, FP8 scales, barriers, reductions and calibration maxima
@@ -125,9 +133,8 @@ __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v 
 // FP32 master (canonical order: per layer W[c_out][3][3][c_in], then b[c_out])
 // -> BF16 B-operand images [tap][c_in group][c_out group][8 c_out][8 c_in] with
 // zero padding, and biases [6][32].
-__global__ void repair_pack_kernel(const float *__restrict__ master, uint16_t *__restrict__ wpack,
-                                   float *__restrict__ bias) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void pack_forward(int e, const float *__restrict__ master, uint16_t *__restrict__ wpack,
+                                             float *__restrict__ bias) {
   if (e < 6 * 32) {
     const int l = e / 32, co = e % 32;
     bias[e] = co < cout(l) ? master[poff(l) + cout(l) * 9 * cin(l) + co] : 0.f;
@@ -147,8 +154,7 @@ __global__ void repair_pack_kernel(const float *__restrict__ master, uint16_t *_
 
 // FP32 master -> the backward's BF16 images of layers 1-5 (see kDPad): element
 // [tap'][c_out group][c_in group][8 c_in][8 c_out] = W[c_out][8 - tap'][c_in].
-__global__ void repair_packT_kernel(const float *__restrict__ master, uint16_t *__restrict__ wpackT) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void pack_backward(int e, const float *__restrict__ master, uint16_t *__restrict__ wpackT) {
   if (e >= kWPackTBytes / 2) return;
   int l = 1;
   while (l < 5 && e >= woffT(l + 1) / 2) ++l;
@@ -160,6 +166,18 @@ __global__ void repair_packT_kernel(const float *__restrict__ master, uint16_t *
   if (co < cout(l) && ci < cin(l)) v = master[poff(l) + (co * 9 + tap) * cin(l) + ci];
   const __nv_bfloat16 h = __float2bfloat16_rn(v);
   wpackT[e] = *reinterpret_cast<const uint16_t *>(&h);
+}
+
+constexpr int kPackThreads = 256;
+constexpr int kPackBlocks = (kWPackBytes / 2 + kPackThreads - 1) / kPackThreads;    // forward images
+constexpr int kPackTBlocks = (kWPackTBytes / 2 + kPackThreads - 1) / kPackThreads;  // backward images
+
+__global__ void __launch_bounds__(kPackThreads) repair_pack_kernel(const float *__restrict__ master,
+                                                                   uint16_t *__restrict__ wpack,
+                                                                   float *__restrict__ bias,
+                                                                   uint16_t *__restrict__ wpackT) {
+  if (blockIdx.x < kPackBlocks) pack_forward(blockIdx.x * kPackThreads + threadIdx.x, master, wpack, bias);
+  else pack_backward((blockIdx.x - kPackBlocks) * kPackThreads + threadIdx.x, master, wpackT);
 }
 
 // ---------------------------------------------------------------- features
@@ -237,7 +255,8 @@ struct NetArgs {
   float *fill;               // [frames][3][H][W], or null
   float *gate;               // [n] mean gate logit per listed tile
   float *out4;               // training: [n][4][16][16] raw outputs, or null
-  uint4 *acts;               // training: [n][6 layer inputs][4 groups][kNPos] (16 B each), or null
+  uint4 *acts;               // training: [n][6 layer inputs][4 groups][kNPos] (16 B each), or null: layer 0's
+                             // group 0 whole, of the others the positions of the M tiles that make them
   uint32_t *amax;            // calibration: [6][32] largest |layer input| (float bits), or null
   uint32_t *status;
 };
@@ -248,7 +267,7 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
   return (lo & 0xffffu) | (hi << 16);
 }
 
-template <bool FP8>
+template <bool FP8, bool KEEP>
 __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(NetArgs a) {
   griddep_wait();
   // BF16: 8 channels per 16-byte group, 4 groups, K = 16 per MMA (two per tap);
@@ -325,12 +344,12 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
                        e4m3x4(bf16_lo(v.z) * is[4], bf16_hi(v.z) * is[5], 0.f, 0.f), 0u, 0u);
       }
       ((uint4 *)bufA)[q] = v;
+      if (KEEP) a.acts[(size_t)t * 6 * 4 * kNPos + q] = v;
       for (int g = 1; g < kGroups; ++g) ((uint4 *)bufA)[g * kNPos + q] = make_uint4(0, 0, 0, 0);
     }
     float gsum = 0.f, gcnt = 0.f;
 #pragma unroll 1
     for (int l = 0; l < 6; ++l) {
-      uint8_t *in = (l & 1) ? bufB : bufA;
       uint8_t *out = (l & 1) ? bufA : bufB;
       const uint32_t sin = (l & 1) ? sB : sA;
       const int ng = ngroups(l), N = ng * 8, MT = mtiles(l);
@@ -341,11 +360,6 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
       umma::fence_before_sync();
       __syncthreads();
       umma::fence_after_sync();
-      if (!FP8 && a.acts) {  // training: keep this layer's input (read beside the MMAs)
-        uint4 *dst = a.acts + ((size_t)t * 6 + l) * 4 * kNPos;
-        const uint4 *srcb = (const uint4 *)in;
-        for (int i = tid; i < kg * kNPos; i += kNetThreads) dst[i] = srcb[i];
-      }
       // lane 0 of warp mt issues the MMAs of M tile mt (the M tiles are issued
       // in parallel) and commits them to barrier mt, so every M tile's epilogue
       // starts as soon as its own accumulator is complete
@@ -425,7 +439,10 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
               uint32_t w4[4];
 #pragma unroll
               for (int j = 0; j < 4; ++j) w4[j] = pack_bf16(v[g * 8 + 2 * j], v[g * 8 + 2 * j + 1]);
-              ((uint4 *)out)[g * kNPos + q] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+              const uint4 hv = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+              ((uint4 *)out)[g * kNPos + q] = hv;
+              // training keeps every layer's input
+              if (KEEP) a.acts[(((size_t)t * 6 + l + 1) * 4 + g) * kNPos + q] = hv;
               if (a.amax && inside && r < kGW - 2 * (l + 1) && c < kGW - 2 * (l + 1)) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -690,8 +707,8 @@ __global__ void __launch_bounds__(1024) repair_sums_kernel(const float *__restri
 __device__ __forceinline__ float psnr_of(float mse) { return mse > 0.f ? -10.f * log10f(mse) : 1e9f; }
 
 // dL/d(output) of the last layer on its 28-wide grid (rows < 16, cols < 16), as
-// the BF16 operand of the backward: channel group 0 holds the 4 outputs, the
-// other groups and every other position are zero
+// the BF16 operand of the backward: channel group 0 (the only one it reads) holds
+// the 4 outputs, zero outside the window
 __global__ void __launch_bounds__(256) repair_dout_kernel(TrainArgs a) {
   const int t = blockIdx.x;
   const uint32_t te = a.tiles[t];
@@ -710,7 +727,7 @@ __global__ void __launch_bounds__(256) repair_dout_kernel(TrainArgs a) {
     a.tile_stats[t * 8 + 6] = label;
   }
   const size_t hw = (size_t)a.W * a.H;
-  for (int q = threadIdx.x; q < kNPos; q += blockDim.x) {
+  for (int q = threadIdx.x; q < kchunks(5) * 16; q += blockDim.x) {
     float g[4] = {0.f, 0.f, 0.f, 0.f};
     const int r = q / kGW, c = q % kGW, y = ty0 + r, x = tx0 + c;
     if (r < kRT && c < kRT && y < a.H && x < a.W) {
@@ -726,67 +743,77 @@ __global__ void __launch_bounds__(256) repair_dout_kernel(TrainArgs a) {
       g[3] = a.lam * (p - label) / ((float)a.n * npx);
     }
     dy[q] = make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), 0u, 0u);
-    for (int grp = 1; grp < 4; ++grp) dy[grp * kNPos + q] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
 // ---------------------------------------------------------------- backward
 struct BwdArgs {
   const uint4 *acts;       // [n][6][4 groups][kNPos]: every layer's BF16 input (forward)
-  const uint4 *dy;         // [n][4][kNPos]: BF16 dL/d(output of layer l), zero outside its window
+  const uint4 *dy;         // [n][4][kNPos]: BF16 dL/d(output of layer l), its c_out groups and the first
+                           // 16 kchunks(l) positions, zero outside the window
   uint4 *dyo;              // [n][4][kNPos]: BF16 dL/d(output of layer l - 1) (l >= 1)
   const uint8_t *wpackT;   // the transposed image of layer l
   float *part;             // [gridDim][cout(l) * 9 * cin(l) + cout(l)] weight and bias gradients per CTA
-  int l, n;
+  int n;
   uint32_t *status;
 };
 
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
 // One layer of the backward pass on the tensor cores; a CTA takes tiles
 // blockIdx.x, + gridDim.x, ... Per tile:
-//   weight gradient: for each tap, D_tap[c_out][c_in] += sum over positions q of
-//     dY[c_out][q] x[c_in][q + shift(tap)]: A = dY^T (K-major, K = positions,
-//     M = 128 rows of which the first c_out are real; the other rows read the next
-//     positions' data and are never used), B = x shifted (MN-major: the 8 c_in of a
-//     position are contiguous), 16 positions per MMA. D_tap stays in tensor
-//     memory across the CTA's tiles and goes to the CTA's partial sums at the end.
 //   input gradient (l >= 1): dX[p][c_in] = sum over tap', c_out of dY[c_out]
 //     [p + shift(tap') - kDPad] W[c_out][8 - tap'][c_in] (the forward's implicit
 //     GEMM on dY stored kDPad positions later), times the ReLU derivative (the
 //     stored input x > 0) inside layer l's input window, stored as BF16 dY of
 //     layer l - 1.
-// Warp 0 issues the weight-gradient MMAs, warp 1 the input-gradient MMAs, each
-// committing to its own barrier; every wait is bounded.
+//   weight gradient: for each tap (dy, s), D[c_out][c_in] += sum over positions c of
+//     dY[c_out][c - s] x[c_in][c + 28 dy]. Both operands are MN-major (a position's
+//     8 channels are contiguous), so dY serves as it is: A's M = 128 rows are the
+//     three copies of dY shifted by s (96 rows; the other 32 read what lies behind
+//     and are never used), B = x moved by dy rows, 16 positions per MMA: three tap
+//     rows make nine taps. D (3 x 32 columns) stays in tensor memory over the CTA's
+//     tiles and goes to its partial sums at the end.
+// Lane 0 of warp mt issues the input gradient's M tile mt, warp kMaxMT's the weight
+// gradient, each committing to a barrier of its own; every wait is bounded. x
+// arrives while the input gradient runs, and the next tile's dY is loaded into
+// registers beside the MMAs.
+template <int L>
 __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   extern __shared__ uint8_t s_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)s_raw + 127) & ~(uintptr_t)127);
-  constexpr int kBuf = 4 * kNPos * 16;
-  uint8_t *bufD = smem;              // dY at positions + kDPad: input-gradient A
-  uint8_t *bufX = smem + kBuf;       // x_l: weight-gradient B, ReLU derivative
-  uint8_t *bufT = smem + 2 * kBuf;   // dY^T [8-position group][c_out group][8 c_out][8 positions]
-  uint8_t *wsm = bufT + kBufT;
+  constexpr int l = L;
+  uint8_t *bufD = smem;            // dY planes
+  uint8_t *bufX = smem + kBufD;    // x_l: weight-gradient B, ReLU derivative
+  uint8_t *wsm = bufX + 4 * kNPos * 16;
   float *s_part = (float *)(wsm + wbytesT(1));  // [8 warps][32]
   float *s_db = s_part + 8 * 32;                // [32] bias gradient over the CTA's tiles
-  uint64_t *mbar = (uint64_t *)(s_db + 32);     // weight gradient, input gradient
-  uint32_t *s_taddr = (uint32_t *)(mbar + 2);
-  const int l = a.l;
+  uint64_t *mbar = (uint64_t *)(s_db + 32);     // input gradient per M tile, weight gradient
+  uint32_t *s_taddr = (uint32_t *)(mbar + kMaxMT + 1);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int wq = wid & 3, wg = wid >> 2;
-  const int ci_n = cin(l), co_n = cout(l);
-  const int NW = l == 0 ? 16 : 32;            // weight-gradient N: c_in padded to 16
-  const int nK = kchunks(l);
-  const int MT = l > 0 ? mtiles(l - 1) : 0;   // input-gradient M tiles: layer l's input window
-  const int vin = kGW - 2 * l, vout = vrows(l);
-  const int kg = kgd(l);
-  constexpr uint32_t kColG = 9 * 32;          // first input-gradient column
+  constexpr int ci_n = cin(l), co_n = cout(l);
+  constexpr int NW = l == 0 ? 16 : 32;            // weight-gradient N: c_in padded to 16
+  constexpr int nK = kchunks(l);
+  constexpr int MT = l > 0 ? mtiles(l - 1) : 0;   // input-gradient M tiles: layer l's input window
+  constexpr int vin = kGW - 2 * l, vout = vrows(l);
+  constexpr int kg = kgd(l);
+  constexpr int gD = (co_n + 7) / 8;                   // c_out groups that are not zero
+  constexpr int gX = l == 0 ? 1 : 4;                   // c_in groups stored
+  constexpr int nX = l == 0 ? kNPos : MT * 128;        // positions of x stored
+  constexpr uint32_t kColG = 3 * 32;                   // first input-gradient column
   {
     if (l > 0) {
       const uint4 *src = (const uint4 *)(a.wpackT + woffT(l));
       for (int i = tid; i < wbytesT(l) / 16; i += kBwdThreads) ((uint4 *)wsm)[i] = src[i];
     }
-    for (int i = tid; i < kBuf / 16; i += kBwdThreads) ((uint4 *)bufD)[i] = make_uint4(0, 0, 0, 0);
-    for (int i = tid; i < kBufT / 16; i += kBwdThreads) ((uint4 *)bufT)[i] = make_uint4(0, 0, 0, 0);
+    // dY's planes and what x leaves out: zero (and finite in the rows nothing reads)
+    uint4 *z = (uint4 *)smem;
+    for (int i = tid; i < (int)kBufD / 16 + 4 * kNPos; i += kBwdThreads) z[i] = make_uint4(0, 0, 0, 0);
     if (tid < 32) s_db[tid] = 0.f;
-    if (tid < 2) umma::mbar_init(mbar + tid, 1);
+    if (tid <= kMaxMT) umma::mbar_init(mbar + tid, 1);
     if (wid == 0) {
       umma::tmem_alloc(s_taddr, kBwdTmemCols);
       umma::tmem_relinquish();
@@ -796,84 +823,89 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     umma::fence_after_sync();
   }
   const uint32_t taddr = *s_taddr;
-  const uint32_t sD = umma::smem_u32(bufD), sX = umma::smem_u32(bufX), sT = umma::smem_u32(bufT),
-                 sW = umma::smem_u32(wsm);
-  uint32_t ph_w = 0, ph_g = 0;
+  const uint32_t sD = umma::smem_u32(bufD), sX = umma::smem_u32(bufX), sW = umma::smem_u32(wsm);
+  uint32_t ph = 0;  // every barrier in use completes once per tile
   bool failed = false, any = false;
+  uint4 dv[gD][kDRegs];  // dY of the tile in hand, then of the next
+  auto load_dy = [&](int t) {
+    const uint4 *ds = a.dy + (size_t)t * 4 * kNPos;
+#pragma unroll
+    for (int g = 0; g < gD; ++g)
+#pragma unroll
+      for (int j = 0; j < kDRegs; ++j) {
+        const int q = tid + j * kBwdThreads;
+        dv[g][j] = q < nK * 16 ? __ldg(ds + g * kNPos + q) : make_uint4(0, 0, 0, 0);
+      }
+  };
+  if ((int)blockIdx.x < a.n) load_dy(blockIdx.x);
   for (int t = blockIdx.x; t < a.n && !failed; t += gridDim.x) {
     // operands of this tile (the previous tile's MMAs have completed)
     const uint4 *xs = a.acts + ((size_t)t * 6 + l) * 4 * kNPos;
-    for (int i = tid; i < 4 * kNPos; i += kBwdThreads) ((uint4 *)bufX)[i] = xs[i];
-    const uint4 *ds = a.dy + (size_t)t * 4 * kNPos;
-    for (int i = tid; i < 4 * nK * 16; i += kBwdThreads) {
-      const int g = i / (nK * 16), q = i % (nK * 16);
-      ((uint4 *)bufD)[g * kNPos + kDPad + q] = ds[g * kNPos + q];
-    }
-    // dY^T: every 8-position x 8-channel block transposed through registers
-    for (int i = tid; i < 2 * nK * 4; i += kBwdThreads) {
-      const int pg = i >> 2, g = i & 3;
-      uint32_t m[8][4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const uint4 v = ds[g * kNPos + pg * 8 + j];
-        m[j][0] = v.x; m[j][1] = v.y; m[j][2] = v.z; m[j][3] = v.w;
-      }
-      uint4 *dst = (uint4 *)(bufT + pg * 512 + g * 128);
+    for (int g = 0; g < gX; ++g)
+      for (int q = tid; q < nX; q += kBwdThreads) cp_async16(sX + (uint32_t)((g * kNPos + q) * 16), xs + g * kNPos + q);
+    asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {  // row c: channel c at the 8 positions
-        uint32_t w[4];
+    for (int g = 0; g < gD; ++g)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t lo = (m[2 * j][c >> 1] >> ((c & 1) * 16)) & 0xffffu;
-          const uint32_t hi = (m[2 * j + 1][c >> 1] >> ((c & 1) * 16)) & 0xffffu;
-          w[j] = lo | (hi << 16);
-        }
-        dst[c] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-    }
-    umma::fence_proxy_async();
-    umma::fence_before_sync();
-    __syncthreads();
-    umma::fence_after_sync();
-    if (lane == 0 && wid == 0) {  // weight gradient: 9 taps x nK MMAs
-      const uint32_t idesc = umma::idesc_bf16(128, NW) | (1u << 16);  // B MN-major
-#pragma unroll 1
-      for (int tap = 0; tap < 9; ++tap) {
-        const int shift = (tap / 3) * kGW + (tap % 3);
-        for (int kc = 0; kc < nK; ++kc) {
-          const uint64_t ad = umma::desc(sT + (uint32_t)(kc * 1024), 512, 128);
-          const uint64_t bd = umma::desc(sX + (uint32_t)((kc * 16 + shift) * 16), 128, kNPos * 16);
-          umma::mma_bf16(taddr + (uint32_t)(tap * NW), ad, bd, idesc, (any || kc > 0) ? 1u : 0u);
+      for (int j = 0; j < kDRegs; ++j) {
+        const int q = tid + j * kBwdThreads;
+        if (q < nK * 16) {
+#pragma unroll
+          for (int s = 0; s < 3; ++s) ((uint4 *)bufD)[(s * 4 + g) * kDPlane + kDPad + s + q] = dv[g][j];
         }
       }
-      umma::mma_commit(mbar + 0);
-    }
-    if (lane == 0 && wid == 1 && l > 0) {  // input gradient: MT tiles x 9 taps x kg / 2 MMAs
-      const uint32_t idesc = umma::idesc_bf16(128, 32);
-      const uint64_t b0 = umma::desc(sW, 4 * 128, 128);
-      for (int mt = 0; mt < MT; ++mt) {
-        const uint64_t a0 = umma::desc(sD + (uint32_t)(mt * 128 * 16), kNPos * 16, 128);
-        const uint32_t d = taddr + kColG + (uint32_t)(mt * 32);
+    if (l > 0) {  // the input gradient needs dY only
+      umma::fence_proxy_async();
+      umma::fence_before_sync();
+      __syncthreads();
+      umma::fence_after_sync();
+      if (lane == 0 && wid < MT) {  // M tile wid: 9 taps x kg / 2 MMAs
+        constexpr uint32_t idesc = umma::idesc_bf16(128, 32);
+        const uint64_t b0 = umma::desc(sW, 4 * 128, 128);
+        const uint64_t a0 = umma::desc(sD + (uint32_t)(wid * 128 * 16), kDPlane * 16, 128);
+        const uint32_t d = taddr + kColG + (uint32_t)(wid * 32);
 #pragma unroll
         for (int tap = 0; tap < 9; ++tap) {
           const int shift = (tap / 3) * kGW + (tap % 3);
+#pragma unroll
           for (int kp = 0; kp < kg / 2; ++kp) {
-            const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kNPos + shift) * 16));
+            const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kDPlane + shift) * 16));
             const uint64_t bd = umma::desc_add(b0, (uint32_t)((tap * kg + 2 * kp) * 4 * 128));
             umma::mma_bf16(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
           }
         }
+        umma::mma_commit(mbar + wid);
       }
-      umma::mma_commit(mbar + 1);
+      __syncwarp();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    umma::fence_proxy_async();
+    umma::fence_before_sync();
+    __syncthreads();
+    umma::fence_after_sync();
+    if (lane == 0 && wid == kMaxMT) {  // weight gradient: 3 tap rows x nK MMAs
+      constexpr uint32_t idesc = umma::idesc_bf16(128, NW) | (1u << 15) | (1u << 16);  // A and B MN-major
+      const uint64_t a0 = umma::desc(sD + (uint32_t)(kDPad * 16), 128, kDPlane * 16);
+      const uint64_t b0 = umma::desc(sX, 128, kNPos * 16);
+#pragma unroll 2
+      for (int kc = 0; kc < nK; ++kc)
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+          umma::mma_bf16(taddr + (uint32_t)(r * NW), umma::desc_add(a0, (uint32_t)(kc * 256)),
+                         umma::desc_add(b0, (uint32_t)((kc * 16 + r * kGW) * 16)), idesc, (any || kc > 0) ? 1u : 0u);
+      umma::mma_commit(mbar + kMaxMT);
     }
     __syncwarp();
     any = true;
+    if (t + (int)gridDim.x < a.n) load_dy(t + (int)gridDim.x);
     // bias gradient: sum of dY over the output window (fixed order per tile)
     {
       const int co = lane;
       float sum = 0.f;
       if (co < co_n) {
-        const uint16_t *col = (const uint16_t *)(bufD + (co >> 3) * kNPos * 16) + (co & 7);
+        const uint16_t *col = (const uint16_t *)(bufD + (co >> 3) * kDPlane * 16) + (co & 7);
+#pragma unroll 8
         for (int q = wid; q < vout * kGW; q += 8) sum += __uint_as_float((uint32_t)col[(kDPad + q) * 8] << 16);
       }
       s_part[wid * 32 + co] = sum;
@@ -887,11 +919,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     }
     bool ok = true;
     if (l > 0) {
-      ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + 1, ph_g));
-      ph_g ^= 1u;
-      umma::fence_after_sync();
       uint4 *dout = a.dyo + (size_t)t * 4 * kNPos;
       for (int mt = wg; mt < MT && ok; mt += 2) {
+        ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + mt, ph));
+        if (!ok) break;
+        umma::fence_after_sync();
         const int q = mt * 128 + wq * 32 + lane;
         const int r = q / kGW, c = q % kGW;
         const bool win = r < vin && c < vin;
@@ -917,70 +949,90 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
           dout[g * kNPos + q] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
         }
       }
-      for (int i = tid; i < 4 * (kNPos - MT * 128); i += kBwdThreads) {
-        const int g = i / (kNPos - MT * 128), q = MT * 128 + i % (kNPos - MT * 128);
-        dout[g * kNPos + q] = make_uint4(0, 0, 0, 0);
-      }
     }
-    // the weight-gradient MMAs read bufT and bufX: wait before the next tile
-    ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + 0, ph_w)) && ok;
-    ph_w ^= 1u;
+    // the weight-gradient MMAs read bufD and bufX: wait before the next tile
+    ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + kMaxMT, ph)) && ok;
     umma::fence_before_sync();
     failed = __syncthreads_or(!ok) != 0;
     umma::fence_after_sync();
+    if (!failed) ph ^= 1u;
   }
   if (failed) {
     if (tid == 0) atomicOr(a.status, kStTimeout);
-    for (int k = 0; k < 2; ++k) umma::mbar_wait(mbar + k, k ? ph_g : ph_w, 1u << 18);
-  } else if (wid == 0) {
-    // weight gradient of the CTA's tiles: TMEM lane = c_out, column = tap * NW + c_in
-    const int npar = co_n * 9 * ci_n;
+    for (int k = 0; k <= kMaxMT; ++k)
+      if (k < MT || k == kMaxMT) umma::mbar_wait(mbar + k, ph, 1u << 18);
+  } else if (wid < 3) {
+    // weight gradient of the CTA's tiles: TMEM lane = s * 32 + c_out, column = dy * NW + c_in
+    constexpr int npar = co_n * 9 * ci_n;
     float *part = a.part + (size_t)blockIdx.x * (npar + co_n);
     const int co = lane;
 #pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
+    for (int r = 0; r < 3; ++r) {
       for (int c16 = 0; c16 < NW / 16; ++c16) {
         float h[16];
         if (any) {
-          umma::tmem_ld16(taddr + (uint32_t)(tap * NW + c16 * 16), h);
+          umma::tmem_ld16(taddr + ((uint32_t)(wid * 32) << 16) + (uint32_t)(r * NW + c16 * 16), h);
         } else {
 #pragma unroll
           for (int i = 0; i < 16; ++i) h[i] = 0.f;
         }
         if (co < co_n)
+#pragma unroll
           for (int i = 0; i < 16; ++i) {
             const int ci = c16 * 16 + i;
-            if (ci < ci_n) part[(co * 9 + tap) * ci_n + ci] = h[i];
+            if (ci < ci_n) part[(co * 9 + r * 3 + wid) * ci_n + ci] = h[i];
           }
       }
     }
-    if (co < co_n) part[npar + co] = s_db[co];
+    if (wid == 0 && co < co_n) part[npar + co] = s_db[co];
   }
   umma::fence_before_sync();
   __syncthreads();
   if (wid == 0) umma::tmem_dealloc(taddr, kBwdTmemCols);
 }
 
-// grad[i] = sum over CTAs (in order) of the partials: deterministic
-__global__ void repair_reduce_kernel(const float *__restrict__ part, int n_parts, int count, float *__restrict__ grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  float sum = 0.f;
-  for (int k = 0; k < n_parts; ++k) sum += part[(size_t)k * count + i];
-  grad[i] = sum;
-}
+struct UpdateArgs {
+  const float *part;  // per layer [n_parts][its parameters], layers in order
+  int n_parts;
+  float *grad, *w, *m, *v;
+  float lr, b1, b2, eps, wd, bc1, bc2;  // AdamW, with lr > 0
+};
 
-__global__ void repair_adamw_kernel(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                                    float *__restrict__ v, int n, float lr, float b1, float b2, float eps, float wd,
-                                    float bc1, float bc2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
-  const float vi = fmaf(b2, v[i], (1.f - b2) * gi * gi);
-  m[i] = mi;
-  v[i] = vi;
-  w[i] -= lr * ((mi / bc1) / (sqrtf(vi / bc2) + eps) + wd * w[i]);
+// grad[i] = sum over the CTAs' partials, deterministic: a block takes 32 parameters,
+// warp w the partials w, w + 8, ... in order, and the warps' sums are added in order.
+// Then AdamW. Bound by the latency of the partials' loads: one thread per parameter
+// with 16 loads in flight took 72 us for 152 CTAs, this 11.
+__global__ void __launch_bounds__(256) repair_update_kernel(UpdateArgs a) {
+  __shared__ float s_sum[8][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  float sum = 0.f;
+  if (i < kRepairParams) {
+    int off = poff(0), end = poff(1);
+#pragma unroll
+    for (int k = 1; k < 6; ++k)
+      if (i >= poff(k)) {
+        off = poff(k);
+        end = poff(k + 1);
+      }
+    const int count = end - off;
+    const float *p = a.part + (size_t)a.n_parts * off + (i - off);
+#pragma unroll 8
+    for (int k = wid; k < a.n_parts; k += 8) sum += __ldg(p + (size_t)k * count);
+  }
+  s_sum[wid][lane] = sum;
+  __syncthreads();
+  if (wid > 0 || i >= kRepairParams) return;
+#pragma unroll
+  for (int w = 1; w < 8; ++w) sum += s_sum[w][lane];
+  a.grad[i] = sum;
+  if (a.lr > 0.f) {
+    const float mi = fmaf(a.b1, a.m[i], (1.f - a.b1) * sum);
+    const float vi = fmaf(a.b2, a.v[i], (1.f - a.b2) * sum * sum);
+    a.m[i] = mi;
+    a.v[i] = vi;
+    a.w[i] -= a.lr * ((mi / a.bc1) / (sqrtf(vi / a.bc2) + a.eps) + a.wd * a.w[i]);
+  }
 }
 
 }  // namespace
@@ -993,27 +1045,36 @@ static int bwd_grid(int n) {
 size_t repair_train_scratch_bytes(int n_tiles) {
   const size_t n = (size_t)(n_tiles > 0 ? n_tiles : 1);
   // activations, raw outputs, gate, two BF16 gradient buffers, tile stats, the
-  // loss sums and the CTAs' partial gradients of one layer
+  // loss sums and the CTAs' partial gradients
   return n * (repair_act_bytes_per_tile() + 4 * kRT * kRT * 4 + 4 + 2 * 4 * kNPos * 16 + 32) +
-         (size_t)bwd_grid((int)n) * kBwdParts * 4 + 10 * 256;  // + alignment of the 8 buffers
+         (size_t)bwd_grid((int)n) * kRepairParams * 4 + 10 * 256;  // + alignment of the 8 buffers
+}
+
+using BwdKernel = void (*)(BwdArgs);
+static BwdKernel bwd_kernel(int l) {
+  static constexpr BwdKernel k[6] = {repair_bwd_kernel<0>, repair_bwd_kernel<1>, repair_bwd_kernel<2>,
+                                     repair_bwd_kernel<3>, repair_bwd_kernel<4>, repair_bwd_kernel<5>};
+  return k[l];
 }
 
 cudaError_t prepare_repair() {
-  cudaError_t e = cudaFuncSetAttribute(repair_net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(repair_net_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)net_smem(false));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(repair_net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)net_smem(true));
+    e = cudaFuncSetAttribute(repair_net_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)net_smem(false));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(repair_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem());
+    e = cudaFuncSetAttribute(repair_net_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)net_smem(true));
+  for (int l = 0; l < 6 && e == cudaSuccess; ++l)
+    e = cudaFuncSetAttribute(bwd_kernel(l), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bwd_smem());
   return e;
 }
 
 cudaError_t repair_pack(const Workspace &ws, cudaStream_t s) {
-  repair_pack_kernel<<<(kWPackBytes / 2 + 255) / 256, 256, 0, s>>>(ws.rp_master, (uint16_t *)ws.rp_wpack,
-                                                                   ws.rp_bias);
-  repair_packT_kernel<<<(kWPackTBytes / 2 + 255) / 256, 256, 0, s>>>(ws.rp_master, (uint16_t *)ws.rp_wpackT);
-  GS_LAUNCHED(2);
+  repair_pack_kernel<<<kPackBlocks + kPackTBlocks, kPackThreads, 0, s>>>(ws.rp_master, (uint16_t *)ws.rp_wpack,
+                                                                         ws.rp_bias, (uint16_t *)ws.rp_wpackT);
+  GS_LAUNCHED(1);
   return cudaGetLastError();
 }
 
@@ -1052,9 +1113,11 @@ cudaError_t repair_forward(const Workspace &ws, const uint4 *feat, int W, int H,
   a.amax = amax;
   a.status = &ws.ctr->status;
   if (fp8) {  // two CTAs per SM fit the FP8 kernel's shared memory
-    launch_k(repair_net_kernel<true>, net_grid(n_max, 2, sm_share), kNetThreads, net_smem(true), s, a);
+    launch_k(repair_net_kernel<true, false>, net_grid(n_max, 2, sm_share), kNetThreads, net_smem(true), s, a);
+  } else if (acts) {
+    launch_k(repair_net_kernel<false, true>, net_grid(n_max, 1, sm_share), kNetThreads, net_smem(false), s, a);
   } else {
-    launch_k(repair_net_kernel<false>, net_grid(n_max, 1, sm_share), kNetThreads, net_smem(false), s, a);
+    launch_k(repair_net_kernel<false, false>, net_grid(n_max, 1, sm_share), kNetThreads, net_smem(false), s, a);
   }
   GS_LAUNCHED(1);
   return cudaGetLastError();
@@ -1114,7 +1177,7 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
   float *stats = (float *)take((size_t)n * 32);
   float *sums = (float *)take(8 * sizeof(float));
   const int G = bwd_grid(n);
-  float *part = (float *)take((size_t)G * kBwdParts * 4);
+  float *part = (float *)take((size_t)G * kRepairParams * 4);
   if ((e = cudaMemsetAsync(sums, 0, 8 * sizeof(float), s)) != cudaSuccess) return e;
   if ((e = repair_forward(ws, b.feat, b.W, b.H, b.tiles, nullptr, (uint32_t)n, nullptr, gate, out4, acts, s, false,
                           nullptr)) != cudaSuccess)
@@ -1139,8 +1202,8 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
   repair_sums_kernel<<<1, 1024, 0, s>>>(stats, n, 5, 6, sums, 2);  // BCE, positive labels
   GS_LAUNCHED(4);
   // backward, last layer first: per layer one tensor-core kernel (weight
-  // gradient into per-CTA partials, input gradient into the other buffer) and
-  // the fixed-order reduction of the partials into this layer's gradient
+  // gradient into per-CTA partials, input gradient into the other buffer); the
+  // update reduces the partials in a fixed order
   uint4 *cur = dy, *nxt = dx;
   for (int l = 5; l >= 0; --l) {
     BwdArgs ba;
@@ -1148,25 +1211,33 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
     ba.dy = cur;
     ba.dyo = nxt;
     ba.wpackT = ws.rp_wpackT;
-    ba.part = part;
-    ba.l = l;
+    ba.part = part + (size_t)G * poff(l);
     ba.n = n;
     ba.status = &ws.ctr->status;
-    repair_bwd_kernel<<<G, kBwdThreads, bwd_smem(), s>>>(ba);
-    const int count = cout(l) * 9 * cin(l) + cout(l);
-    repair_reduce_kernel<<<(count + 255) / 256, 256, 0, s>>>(part, G, count, ws.rp_grad + poff(l));
-    GS_LAUNCHED(2);
+    bwd_kernel(l)<<<G, kBwdThreads, bwd_smem(), s>>>(ba);
+    GS_LAUNCHED(1);
     uint4 *tmp = cur;
     cur = nxt;
     nxt = tmp;
   }
-  if (o.lr > 0.f) {
-    repair_adamw_kernel<<<(kRepairParams + 255) / 256, 256, 0, s>>>(
-        ws.rp_master, ws.rp_grad, ws.rp_m, ws.rp_v, kRepairParams, o.lr, o.beta1, o.beta2, o.eps, o.weight_decay,
-        1.f - powf(o.beta1, (float)o.step), 1.f - powf(o.beta2, (float)o.step));
-    GS_LAUNCHED(1);
+  UpdateArgs u;
+  u.part = part;
+  u.n_parts = G;
+  u.grad = ws.rp_grad;
+  u.w = ws.rp_master;
+  u.m = ws.rp_m;
+  u.v = ws.rp_v;
+  u.lr = o.lr;
+  u.b1 = o.beta1;
+  u.b2 = o.beta2;
+  u.eps = o.eps;
+  u.wd = o.weight_decay;
+  u.bc1 = 1.f - powf(o.beta1, (float)o.step);
+  u.bc2 = 1.f - powf(o.beta2, (float)o.step);
+  repair_update_kernel<<<(kRepairParams + 31) / 32, 256, 0, s>>>(u);
+  GS_LAUNCHED(1);
+  if (o.lr > 0.f)
     if ((e = repair_pack(ws, s)) != cudaSuccess) return e;
-  }
   if (host_loss) {
     float h[8];
     if ((e = cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s)) != cudaSuccess) return e;
