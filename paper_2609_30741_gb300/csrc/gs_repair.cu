@@ -46,8 +46,9 @@ constexpr int kRT = 16;                 // output tile edge
 constexpr int kHalo = 6;                // receptive-field radius of six 3x3 layers
 constexpr int kGW = kRT + 2 * kHalo;    // 28: width of the position grid
 constexpr int kNPos = 832;              // positions per activation buffer (6 M tiles + tap reach)
-constexpr int kNetThreads = 256;  // two warpgroups take alternate M tiles of the epilogue
-constexpr int kTmemCols = 256;
+constexpr int kNetWorkers = 256;                // two warpgroups take alternate M tiles of the epilogue
+constexpr int kNetThreads = kNetWorkers + 32;  // and one warp issues the MMAs
+constexpr int kTmemCols = 256;  // 6 M tiles x 32, and the last layer's 4 x 16 beside them
 
 __host__ __device__ constexpr int cin(int l) { return l == 0 ? 6 : 32; }
 __host__ __device__ constexpr int cout(int l) { return l == 5 ? 4 : 32; }
@@ -68,6 +69,7 @@ __host__ __device__ constexpr int mtiles(int l) { return ((kGW - 2 * (l + 1)) * 
 
 constexpr int kMaxMT = 6;  // M tiles of the widest layer
 constexpr int kWPackBytes = woff(6);
+static_assert(kMaxMT * 32 + mtiles(5) * 16 <= kTmemCols, "tensor memory of the network");
 static_assert(kWPackBytes == 92160, "packed weight image size");
 // FP8 images: [tap][2 c_in groups of 16][c_out groups][8][16 B]
 __host__ __device__ constexpr int wbytes8(int l) { return 9 * 2 * ngroups(l) * 128; }
@@ -80,7 +82,6 @@ constexpr int kWPack8Bytes = woff8(6);
 static_assert(kWPack8Bytes == 50688, "packed FP8 weight image size");
 static_assert(poff(6) == kRepairParams, "parameter count");
 static_assert(mtiles(0) <= kMaxMT, "M tiles per layer");
-static_assert(kMaxMT <= kNetThreads / 32, "one issuing warp per M tile");
 // backward: the input gradient of layer l (l >= 1) convolves dY_l, stored kDPad
 // positions later in shared memory, with the flipped transposed weights
 // W'[tap'][c_out group][c_in group][8 c_in][8 c_out] (W' at tap' = W at 8 - tap')
@@ -96,7 +97,8 @@ constexpr int kWPackTBytes = woffT(6);
 static_assert(kWPackTBytes == 82944, "packed transposed weight image size");
 __host__ __device__ constexpr int vrows(int l) { return kGW - 2 * (l + 1); }            // layer l's output edge
 __host__ __device__ constexpr int kchunks(int l) { return (vrows(l) * kGW + 15) / 16; }  // weight-gradient K = 16 steps
-constexpr int kBwdThreads = 256;
+constexpr int kBwdWorkers = 256;               // stage operands, read the accumulators back
+constexpr int kBwdThreads = kBwdWorkers + 32;  // and the warp that issues the MMAs
 constexpr int kBwdTmemCols = 512;   // 3 tap rows x 32 (weight gradient) + 6 M tiles x 32 (input gradient)
 // dY in shared memory: planes [horizontal tap s][c_out group] of kDPlane positions,
 // dY at position q stored kDPad + s + q into its plane, zero elsewhere
@@ -104,14 +106,14 @@ constexpr int kDPlane = 800;
 constexpr int kDRegs = 3;  // positions of a plane a thread stages
 static_assert(3 * 32 + kMaxMT * 32 <= kBwdTmemCols, "tensor memory of the backward");
 static_assert(kchunks(0) * 16 + 2 * kGW + 2 <= kNPos, "weight gradient: reach of x");
-static_assert(kDPad + 2 + kchunks(0) * 16 <= kDPlane && kchunks(0) * 16 <= kDRegs * kBwdThreads, "a plane holds dY");
+static_assert(kDPad + 2 + kchunks(0) * 16 <= kDPlane && kchunks(0) * 16 <= kDRegs * kBwdWorkers, "a plane holds dY");
 // the input gradient reads dY at positions < kDPad + vin * 28 of a plane, its unused rows a little of the next;
 // 16 groups of M = 128 rows read 4 planes past the 12
 static_assert(vrows(0) * kGW + kDPad <= kDPlane && kMaxMT * 128 + kDPad <= kDPlane + kDPad, "input gradient: reach of dY");
 constexpr size_t kBufD = 12 * (size_t)kDPlane * 16;
 static_assert(4 * (size_t)kDPlane * 16 <= 4 * (size_t)kNPos * 16, "reach of the unused rows");
 __host__ __device__ constexpr size_t bwd_smem() {
-  return 128 + kBufD + 4 * (size_t)kNPos * 16 + wbytesT(1) + (8 * 32 + 32) * 4 + (kMaxMT + 1) * 8 + 16;
+  return 128 + kBufD + 4 * (size_t)kNPos * 16 + wbytesT(1) + (8 * 32 + 32) * 4 + (kMaxMT + 2) * 8 + 16;
 }
 static_assert(bwd_smem() <= 227 * 1024, "shared memory of the backward");
 static_assert(kMaxMT * 128 + 2 * kGW + 2 <= kNPos, "activation buffer reach");
@@ -119,7 +121,7 @@ static_assert(kMaxMT * 128 + 2 * kGW + 2 <= kNPos, "activation buffer reach");
 // bias, FP8 scales, barriers, reductions and calibration maxima
 __host__ __device__ constexpr size_t net_smem(bool fp8) {
   return 128 + 2 * (size_t)((fp8 ? 2 : 4) * kNPos * 16) + (fp8 ? kWPack8Bytes : kWPackBytes) + 3 * 6 * 32 * 4 +
-         8 * kMaxMT + 4 + 16 * 4 + 6 * 32 * 4 + 64;
+         8 * (2 * kMaxMT + mtiles(5) + 3) + 4 + 32 * 4 + 6 * 32 * 4 + 64;
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -267,8 +269,21 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
   return (lo & 0xffffu) | (hi << 16);
 }
 
+// The last warp issues every MMA in order, M tile by M tile and layer by layer; the
+// workers read an M tile back as soon as it is complete and release its positions to
+// the next layer, whose M tile mt needs those of mt and mt + 1 (the taps reach 58
+// positions on). So the tensor core works on while earlier M tiles are read back, and
+// there is no barrier between layers. What an epilogue overwrites has been read: it
+// writes M tile mt of the buffer that the layer before read at mt and mt - 1, whose
+// MMAs completed before the M tile it reads. The next tile's input is stored and its
+// first layer starts while the last layer, in columns of its own, is read back.
+// Bound by the MMAs (M = 128, N = 32, K = 16 or 32: 41 cycles each) for BF16, by the
+// epilogues' latency for FP8 (two CTAs per SM). 1000 tiles BF16: 156 -> 101 us, 2600
+// tiles FP8: 238 -> 210 us (each M tile issued by a warp of its own, a barrier per layer
+// before). 96 registers: the kernel runs beside the ROI binning, which at 158 took 10 us
+// longer a frame (1.5M surfels, 1080p).
 template <bool FP8, bool KEEP>
-__global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(NetArgs a) {
+__global__ void __launch_bounds__(kNetThreads, KEEP ? 1 : 2) repair_net_kernel(NetArgs a) {
   griddep_wait();
   // BF16: 8 channels per 16-byte group, 4 groups, K = 16 per MMA (two per tap);
   // FP8: 16 channels per group, 2 groups, K = 32 per MMA (one per tap)
@@ -276,6 +291,7 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
   constexpr int kGroups = 32 / kChPerGroup;
   constexpr int kBuf = kGroups * kNPos * 16;
   constexpr int kWBytes = FP8 ? kWPack8Bytes : kWPackBytes;
+  constexpr int kIn = (kNPos + kNetWorkers - 1) / kNetWorkers;  // input positions per worker
   extern __shared__ uint8_t s_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)s_raw + 127) & ~(uintptr_t)127);
   uint8_t *bufA = smem;
@@ -284,11 +300,16 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
   float *s_bias = (float *)(wsm + kWBytes);
   float *s_sw = s_bias + 6 * 32;        // FP8: weight scales
   float *s_isx = s_sw + 6 * 32;         // FP8: reciprocal input scales
-  uint64_t *mbar = (uint64_t *)(s_isx + 6 * 32);  // one per M tile of a layer
-  uint32_t *s_taddr = (uint32_t *)(mbar + kMaxMT);
-  float *s_red = (float *)(s_taddr + 1);          // [8 warps][2]
-  uint32_t *s_amax = (uint32_t *)(s_red + 16);    // [6][32] calibration maxima
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  uint64_t *done = (uint64_t *)(s_isx + 6 * 32);  // per M tile: its accumulator is complete
+  uint64_t *ready = done + kMaxMT;                // per M tile: read back, the next layer's input written
+  uint64_t *done5 = ready + kMaxMT;               // as done, for the last layer
+  uint64_t *loaded = done5 + mtiles(5);            // the tile's first input is written
+  uint64_t *summed = loaded + 1;                  // the warps' gate sums are written
+  uint64_t *drained = summed + 1;                 // after a failure: nothing is in flight
+  uint32_t *s_taddr = (uint32_t *)(drained + 1);
+  float *s_red = (float *)(s_taddr + 1);          // [2 tiles in turn][8 warps][2]
+  uint32_t *s_amax = (uint32_t *)(s_red + 32);    // [6][32] calibration maxima
+  const int tid = threadIdx.x, lane = tid & 31, wid = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int wq = wid & 3, wg = wid >> 2;  // TMEM lane quarter of the warp; its warpgroup
   const uint32_t n = load_n(a.n_tiles, a.n_max);
   if (blockIdx.x >= n) return;
@@ -308,217 +329,269 @@ __global__ void __launch_bounds__(kNetThreads, FP8 ? 2 : 1) repair_net_kernel(Ne
     }
     uint4 *z = (uint4 *)smem;
     for (int i = tid; i < 2 * kBuf / 16; i += kNetThreads) z[i] = make_uint4(0, 0, 0, 0);
-    if (tid < kMaxMT) umma::mbar_init(mbar + tid, 1);
+    if (tid < kMaxMT) {
+      umma::mbar_init(done + tid, 1);
+      umma::mbar_init(ready + tid, kNetWorkers / 2);
+    }
+    if (tid < mtiles(5)) umma::mbar_init(done5 + tid, 1);
+    if (tid == 0) {
+      umma::mbar_init(loaded, kNetWorkers);
+      umma::mbar_init(summed, kNetWorkers / 32);
+      umma::mbar_init(drained, 1);
+    }
     if (wid == 0) {
       umma::tmem_alloc(s_taddr, kTmemCols);
       umma::tmem_relinquish();
     }
+    umma::fence_proxy_async();
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
   }
   const uint32_t taddr = *s_taddr;
   const uint32_t sA = umma::smem_u32(bufA), sB = umma::smem_u32(bufB), sW = umma::smem_u32(wsm);
-  uint32_t phases = 0;  // bit mt: parity the next completion of mbar[mt] flips to
-  bool failed = false;
+  bool ok = true;  // the same on every lane of a warp
 
-  for (uint32_t t = blockIdx.x; t < n && !failed; t += gridDim.x) {
-    const uint32_t te = a.tiles[t];
-    const int frame = (int)(te >> 24), ty0 = (int)((te >> 12) & 0xfffu) * kRT, tx0 = (int)(te & 0xfffu) * kRT;
-    const uint4 *fin = a.feat + (size_t)frame * a.W * a.H;
-    // layer-1 input: the 28x28 feature window (zeros outside the image); the
-    // 6 features + zeros fill channel group 0, the other groups are zero (K padding)
-    for (int q = tid; q < kNPos; q += kNetThreads) {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (q < kGW * kGW) {
-        const int y = ty0 - kHalo + q / kGW, x = tx0 - kHalo + q % kGW;
-        if (y >= 0 && y < a.H && x >= 0 && x < a.W) v = fin[(size_t)y * a.W + x];
-      }
-      if (a.amax) {
-        const float f[6] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z)};
-        for (int c = 0; c < 6; ++c) atomicMax(&s_amax[c], __float_as_uint(fabsf(f[c])));
-      }
-      if (FP8) {
-        const float *is = s_isx;  // layer-0 input scales
-        v = make_uint4(e4m3x4(bf16_lo(v.x) * is[0], bf16_hi(v.x) * is[1], bf16_lo(v.y) * is[2], bf16_hi(v.y) * is[3]),
-                       e4m3x4(bf16_lo(v.z) * is[4], bf16_hi(v.z) * is[5], 0.f, 0.f), 0u, 0u);
-      }
-      ((uint4 *)bufA)[q] = v;
-      if (KEEP) a.acts[(size_t)t * 6 * 4 * kNPos + q] = v;
-      for (int g = 1; g < kGroups; ++g) ((uint4 *)bufA)[g * kNPos + q] = make_uint4(0, 0, 0, 0);
-    }
-    float gsum = 0.f, gcnt = 0.f;
+  if (wid == kNetWorkers / 32) {  // ---- the issuing warp
+    uint32_t ph = 0, ph_l = 0;    // bit mt: parity of ready[mt]; of loaded
+    for (uint32_t t = blockIdx.x; t < n && ok; t += gridDim.x) {
+      ok = __all_sync(0xffffffffu, umma::mbar_wait(loaded, ph_l));
+      ph_l ^= 1u;
+#pragma unroll
+      for (int l = 0; l < 6; ++l) {
+        const uint32_t sin = (l & 1) ? sB : sA;
+        const int ng = ngroups(l), N = ng * 8, MT = mtiles(l);
+        const int kg = FP8 ? 2 : kgroups(l);  // 16-byte K groups of this layer's input
+        const uint32_t idesc = FP8 ? umma::idesc_e4m3(128, N) : umma::idesc_bf16(128, N);
+        const uint64_t a00 = umma::desc(sin, kNPos * 16, 128);
+        const uint64_t b0 = umma::desc(sW + (uint32_t)(FP8 ? woff8(l) : woff(l)), ng * 128, 128);
+        const int before = l > 0 ? mtiles(l - 1) : 0;  // the M tiles that wrote the input
+        int have = 0;                                  // of which are written
 #pragma unroll 1
-    for (int l = 0; l < 6; ++l) {
-      uint8_t *out = (l & 1) ? bufA : bufB;
-      const uint32_t sin = (l & 1) ? sB : sA;
-      const int ng = ngroups(l), N = ng * 8, MT = mtiles(l);
-      const int kg = FP8 ? 2 : kgroups(l);  // 16-byte K groups of this layer's input
-      // this layer's input (written by all threads) is complete and visible to
-      // the tensor core
+        for (int mt = 0; mt < MT && ok; ++mt) {
+          for (; have < before && have < mt + 2 && ok; ++have) {
+            ok = __all_sync(0xffffffffu, umma::mbar_wait(ready + have, (ph >> have) & 1u));
+            ph ^= 1u << have;
+          }
+          umma::fence_after_sync();
+          if (ok && umma::elect()) {
+            const uint64_t a0 = umma::desc_add(a00, (uint32_t)(mt * 128 * 16));
+            const uint32_t d = taddr + (uint32_t)(l < 5 ? mt * 32 : kMaxMT * 32 + mt * 16);
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+              const int shift = (tap / 3) * kGW + (tap % 3);
+#pragma unroll
+              for (int kp = 0; kp < kg / 2; ++kp) {  // two 16-byte groups per MMA
+                const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kNPos + shift) * 16));
+                const uint64_t bd = umma::desc_add(b0, (uint32_t)((tap * kg + 2 * kp) * ng * 128));
+                if (FP8) umma::mma_e4m3(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
+                else umma::mma_bf16(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
+              }
+            }
+            umma::mma_commit((l < 5 ? done : done5) + mt);
+          }
+          __syncwarp();
+        }
+      }
+    }
+  } else {  // ---- the workers
+    uint4 vin[kIn];
+    auto fetch = [&](uint32_t te) {  // the tile's 28x28 feature window (zeros outside the image)
+      const int frame = (int)(te >> 24), ty0 = (int)((te >> 12) & 0xfffu) * kRT, tx0 = (int)(te & 0xfffu) * kRT;
+      const uint4 *fin = a.feat + (size_t)frame * a.W * a.H;
+#pragma unroll
+      for (int j = 0; j < kIn; ++j) {
+        const int q = tid + j * kNetWorkers;
+        vin[j] = make_uint4(0, 0, 0, 0);
+        const int y = ty0 - kHalo + q / kGW, x = tx0 - kHalo + q % kGW;
+        if (q < kGW * kGW && y >= 0 && y < a.H && x >= 0 && x < a.W) vin[j] = fin[(size_t)y * a.W + x];
+      }
+    };
+    // layer 0's input: the 6 features + zeros fill channel group 0, group 1 is zero (K padding)
+    auto store_input = [&](uint32_t t) {
+#pragma unroll
+      for (int j = 0; j < kIn; ++j) {
+        const int q = tid + j * kNetWorkers;
+        if (q >= kNPos) break;
+        uint4 v = vin[j];
+        if (a.amax) {
+          const float f[6] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y), bf16_lo(v.z), bf16_hi(v.z)};
+          for (int c = 0; c < 6; ++c) atomicMax(&s_amax[c], __float_as_uint(fabsf(f[c])));
+        }
+        if (FP8) {
+          const float *is = s_isx;  // layer-0 input scales
+          v = make_uint4(e4m3x4(bf16_lo(v.x) * is[0], bf16_hi(v.x) * is[1], bf16_lo(v.y) * is[2], bf16_hi(v.y) * is[3]),
+                         e4m3x4(bf16_lo(v.z) * is[4], bf16_hi(v.z) * is[5], 0.f, 0.f), 0u, 0u);
+        }
+        ((uint4 *)bufA)[q] = v;
+        ((uint4 *)bufA)[kNPos + q] = make_uint4(0, 0, 0, 0);
+        if (KEEP) a.acts[(size_t)t * 6 * 4 * kNPos + q] = v;
+      }
       umma::fence_proxy_async();
       umma::fence_before_sync();
-      __syncthreads();
-      umma::fence_after_sync();
-      // lane 0 of warp mt issues the MMAs of M tile mt (the M tiles are issued
-      // in parallel) and commits them to barrier mt, so every M tile's epilogue
-      // starts as soon as its own accumulator is complete
-      if (lane == 0 && wid < MT) {
-        const int mt = wid;
-        const uint32_t idesc = FP8 ? umma::idesc_e4m3(128, N) : umma::idesc_bf16(128, N);
-        const uint32_t wl = sW + (uint32_t)(FP8 ? woff8(l) : woff(l));
-        const uint64_t a0 = umma::desc(sin + (uint32_t)(mt * 128 * 16), kNPos * 16, 128);
-        const uint64_t b0 = umma::desc(wl, ng * 128, 128);
-        const uint32_t d = taddr + (uint32_t)(mt * N);
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const int shift = (tap / 3) * kGW + (tap % 3);
-          for (int kp = 0; kp < kg / 2; ++kp) {  // two 16-byte groups per MMA
-            const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kNPos + shift) * 16));
-            const uint64_t bd = umma::desc_add(b0, (uint32_t)((tap * kg + 2 * kp) * ng * 128));
-            if (FP8) umma::mma_e4m3(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
-            else umma::mma_bf16(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
-          }
+      umma::mbar_arrive(loaded);
+    };
+    uint32_t ph = 0, ph5 = 0, ph_s = 0;  // bit mt: parity of done[mt]; of done5, summed
+    int turn = 0;
+    uint32_t te = a.tiles[blockIdx.x];
+    fetch(te);
+    store_input(blockIdx.x);
+    for (uint32_t t = blockIdx.x; t < n && ok; t += gridDim.x) {
+      const int frame = (int)(te >> 24), ty0 = (int)((te >> 12) & 0xfffu) * kRT, tx0 = (int)(te & 0xfffu) * kRT;
+      const uint4 *fin = a.feat + (size_t)frame * a.W * a.H;
+      const uint32_t tn = t + gridDim.x;
+      const uint32_t te_next = tn < n ? a.tiles[tn] : 0u;
+      float gsum = 0.f, gcnt = 0.f;
+#pragma unroll 1
+      for (int l = 0; l < 6 && ok; ++l) {
+        uint8_t *out = (l & 1) ? bufA : bufB;
+        const int MT = mtiles(l);
+        if (l == 4 && tn < n) fetch(te_next);
+        if (l == 5) {
+          // an M tile of this layer is complete, and with it every MMA of layer 4 on the
+          // buffer that takes the next tile
+          ok = __all_sync(0xffffffffu, umma::mbar_wait(done5 + wg, ph5));
+          if (!ok) break;
+          if (tn < n) store_input(tn);
         }
-        umma::mma_commit(mbar + mt);
-      }
-      __syncwarp();
-      // epilogue: accumulator rows -> scale, bias, ReLU, border zeroing -> next buffer
-      const int shiftL = l + 1;  // this layer's output grid starts (l + 1) pixels in
-      bool layer_ok = true;
-      for (int mt = 0; mt < MT; ++mt) {
-        // warpgroup mt % 2 reads M tile mt; every thread tracks every barrier's phase
-        const uint32_t par = (phases >> mt) & 1u;
-        phases ^= 1u << mt;
-        if ((mt & 1) != wg) continue;
-        // the same decision on every lane of the warp (tcgen05.ld is warp-wide)
-        const bool ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + mt, par));
-        if (!ok) {
-          layer_ok = false;
-          break;
-        }
-        umma::fence_after_sync();
-        const int q = mt * 128 + wq * 32 + lane;
-        const int r = q / kGW, c = q % kGW;
-        const int y = ty0 - kHalo + shiftL + r, x = tx0 - kHalo + shiftL + c;
-        const bool inside = y >= 0 && y < a.H && x >= 0 && x < a.W;
-        const uint32_t tl = taddr + ((uint32_t)(wq * 32) << 16) + (uint32_t)(mt * N);
-        const float *bl = s_bias + l * 32;
-        const float *swl = s_sw + l * 32;
-        if (l < 5) {
-          float v[32];
-          float h[16];
-          umma::tmem_ld16(tl, h);
+        // epilogue: accumulator rows -> scale, bias, ReLU, border zeroing -> next buffer
+        const int shiftL = l + 1;  // this layer's output grid starts (l + 1) pixels in
+        for (int mt = wg; mt < MT; mt += 2) {
+          // the same decision on every lane of the warp (tcgen05.ld is warp-wide)
+          ok = __all_sync(0xffffffffu, l < 5 ? umma::mbar_wait(done + mt, (ph >> mt) & 1u)
+                                             : umma::mbar_wait(done5 + mt, ph5));
+          if (!ok) break;
+          if (l < 5) ph ^= 1u << mt;
+          umma::fence_after_sync();
+          const int q = mt * 128 + wq * 32 + lane;
+          const int r = q / kGW, c = q % kGW;
+          const int y = ty0 - kHalo + shiftL + r, x = tx0 - kHalo + shiftL + c;
+          const bool inside = y >= 0 && y < a.H && x >= 0 && x < a.W;
+          const uint32_t tl =
+              taddr + ((uint32_t)(wq * 32) << 16) + (uint32_t)(l < 5 ? mt * 32 : kMaxMT * 32 + mt * 16);
+          const float *bl = s_bias + l * 32;
+          const float *swl = s_sw + l * 32;
+          if (l < 5) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = h[i];
-          umma::tmem_ld16(tl + 16, h);
+            for (int hf = 0; hf < 2; ++hf) {  // 16 channels at a time
+              float v[16];
+              umma::tmem_ld16(tl + 16 * hf, v);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[16 + i] = h[i];
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float yv = FP8 ? fmaf(v[i], swl[i], bl[i]) : v[i] + bl[i];
-            v[i] = inside ? fmaxf(yv, 0.f) : 0.f;
-          }
-          if (FP8) {
-            const float *is = s_isx + (l + 1) * 32;  // next layer's input scales
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-              const int o = g * 16;
-              ((uint4 *)out)[g * kNPos + q] =
-                  make_uint4(e4m3x4(v[o] * is[o], v[o + 1] * is[o + 1], v[o + 2] * is[o + 2], v[o + 3] * is[o + 3]),
-                             e4m3x4(v[o + 4] * is[o + 4], v[o + 5] * is[o + 5], v[o + 6] * is[o + 6],
-                                    v[o + 7] * is[o + 7]),
-                             e4m3x4(v[o + 8] * is[o + 8], v[o + 9] * is[o + 9], v[o + 10] * is[o + 10],
-                                    v[o + 11] * is[o + 11]),
-                             e4m3x4(v[o + 12] * is[o + 12], v[o + 13] * is[o + 13], v[o + 14] * is[o + 14],
-                                    v[o + 15] * is[o + 15]));
-            }
-          } else {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              uint32_t w4[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) w4[j] = pack_bf16(v[g * 8 + 2 * j], v[g * 8 + 2 * j + 1]);
-              const uint4 hv = make_uint4(w4[0], w4[1], w4[2], w4[3]);
-              ((uint4 *)out)[g * kNPos + q] = hv;
-              // training keeps every layer's input
-              if (KEEP) a.acts[(((size_t)t * 6 + l + 1) * 4 + g) * kNPos + q] = hv;
-              if (a.amax && inside && r < kGW - 2 * (l + 1) && c < kGW - 2 * (l + 1)) {
+              for (int i = 0; i < 16; i += 4) {
+                const float4 b4 = *(const float4 *)(bl + hf * 16 + i);
+                const float4 s4 = FP8 ? *(const float4 *)(swl + hf * 16 + i) : make_float4(1.f, 1.f, 1.f, 1.f);
+                const float bb[4] = {b4.x, b4.y, b4.z, b4.w}, ss[4] = {s4.x, s4.y, s4.z, s4.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                  atomicMax(&s_amax[(l + 1) * 32 + g * 8 + 2 * j], w4[j] << 16);
-                  atomicMax(&s_amax[(l + 1) * 32 + g * 8 + 2 * j + 1], w4[j] & 0xffff0000u);
+                  const float yv = FP8 ? fmaf(v[i + j], ss[j], bb[j]) : v[i + j] + bb[j];
+                  v[i + j] = inside ? fmaxf(yv, 0.f) : 0.f;
+                }
+              }
+              if (FP8) {
+                const float4 *is = (const float4 *)(s_isx + (l + 1) * 32 + hf * 16);  // next layer's input scales
+                uint32_t w4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                  const float4 f = is[j];
+                  w4[j] = e4m3x4(v[4 * j] * f.x, v[4 * j + 1] * f.y, v[4 * j + 2] * f.z, v[4 * j + 3] * f.w);
+                }
+                ((uint4 *)out)[hf * kNPos + q] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+              } else {
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                  const int g = hf * 2 + k;
+                  uint32_t w4[4];
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) w4[j] = pack_bf16(v[k * 8 + 2 * j], v[k * 8 + 2 * j + 1]);
+                  const uint4 hv = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+                  ((uint4 *)out)[g * kNPos + q] = hv;
+                  if (a.amax && inside && r < kGW - 2 * (l + 1) && c < kGW - 2 * (l + 1)) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                      atomicMax(&s_amax[(l + 1) * 32 + g * 8 + 2 * j], w4[j] << 16);
+                      atomicMax(&s_amax[(l + 1) * 32 + g * 8 + 2 * j + 1], w4[j] & 0xffff0000u);
+                    }
+                  }
+                  // training keeps every layer's input
+                  if (KEEP) a.acts[(((size_t)t * 6 + l + 1) * 4 + g) * kNPos + q] = hv;
                 }
               }
             }
-          }
-        } else {
-          float v[16];
-          umma::tmem_ld16(tl, v);
-          if (r < kRT && c < kRT) {
-            const float o0 = FP8 ? fmaf(v[0], swl[0], bl[0]) : v[0] + bl[0];
-            const float o1 = FP8 ? fmaf(v[1], swl[1], bl[1]) : v[1] + bl[1];
-            const float o2 = FP8 ? fmaf(v[2], swl[2], bl[2]) : v[2] + bl[2];
-            const float o3 = FP8 ? fmaf(v[3], swl[3], bl[3]) : v[3] + bl[3];
-            if (a.out4) {
-              float *o = a.out4 + (size_t)t * 4 * kRT * kRT + r * kRT + c;
-              o[0] = o0;
-              o[kRT * kRT] = o1;
-              o[2 * kRT * kRT] = o2;
-              o[3 * kRT * kRT] = o3;
-            }
-            if (inside) {
-              if (a.fill) {  // the network corrects the method's fill (feature RGB)
-                const size_t hw = (size_t)a.W * a.H;
-                const uint4 fv = fin[(size_t)y * a.W + x];
-                float *f = a.fill + (size_t)frame * 3 * hw + (size_t)y * a.W + x;
-                f[0] = bf16_lo(fv.x) + o0;
-                f[hw] = bf16_hi(fv.x) + o1;
-                f[2 * hw] = bf16_lo(fv.y) + o2;
+            umma::fence_proxy_async();
+            umma::fence_before_sync();
+            umma::mbar_arrive(ready + mt);
+          } else {
+            float v[16];
+            umma::tmem_ld16(tl, v);
+            if (r < kRT && c < kRT) {
+              const float o0 = FP8 ? fmaf(v[0], swl[0], bl[0]) : v[0] + bl[0];
+              const float o1 = FP8 ? fmaf(v[1], swl[1], bl[1]) : v[1] + bl[1];
+              const float o2 = FP8 ? fmaf(v[2], swl[2], bl[2]) : v[2] + bl[2];
+              const float o3 = FP8 ? fmaf(v[3], swl[3], bl[3]) : v[3] + bl[3];
+              if (a.out4) {
+                float *o = a.out4 + (size_t)t * 4 * kRT * kRT + r * kRT + c;
+                o[0] = o0;
+                o[kRT * kRT] = o1;
+                o[2 * kRT * kRT] = o2;
+                o[3 * kRT * kRT] = o3;
               }
-              gsum += o3;
-              gcnt += 1.f;
+              if (inside) {
+                if (a.fill) {  // the network corrects the method's fill (feature RGB)
+                  const size_t hw = (size_t)a.W * a.H;
+                  const uint4 fv = fin[(size_t)y * a.W + x];
+                  float *f = a.fill + (size_t)frame * 3 * hw + (size_t)y * a.W + x;
+                  f[0] = bf16_lo(fv.x) + o0;
+                  f[hw] = bf16_hi(fv.x) + o1;
+                  f[2 * hw] = bf16_lo(fv.y) + o2;
+                }
+                gsum += o3;
+                gcnt += 1.f;
+              }
             }
           }
         }
       }
-      umma::fence_before_sync();
-      failed = __syncthreads_or(!layer_ok) != 0;  // the same decision on every thread
-      if (failed) {
-        if (tid == 0) atomicOr(a.status, kStTimeout);
-        break;
-      }
-    }
-    if (failed) break;
-    // gate logit: mean over the tile's pixels inside the image
+      if (!ok) break;
+      ph5 ^= 1u;
+      te = te_next;
+      // gate logit: mean over the tile's pixels inside the image
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
-      gcnt += __shfl_xor_sync(0xffffffffu, gcnt, o);
-    }
-    if (lane == 0) {
-      s_red[wid * 2] = gsum;
-      s_red[wid * 2 + 1] = gcnt;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      float sm = 0.f, cn = 0.f;
-      for (int w = 0; w < kNetThreads / 32; ++w) {
-        sm += s_red[2 * w];
-        cn += s_red[2 * w + 1];
+      for (int o = 16; o > 0; o >>= 1) {
+        gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
+        gcnt += __shfl_xor_sync(0xffffffffu, gcnt, o);
       }
-      a.gate[t] = cn > 0.f ? sm / cn : 0.f;
+      float *red = s_red + turn * 16;
+      turn ^= 1;
+      if (lane == 0) {
+        red[wid * 2] = gsum;
+        red[wid * 2 + 1] = gcnt;
+        umma::mbar_arrive(summed);
+      }
+      if (wid == 0) {
+        ok = __all_sync(0xffffffffu, umma::mbar_wait(summed, ph_s));
+        ph_s ^= 1u;
+        if (ok && lane == 0) {
+          float sm = 0.f, cn = 0.f;
+          for (int w = 0; w < kNetWorkers / 32; ++w) {
+            sm += red[2 * w];
+            cn += red[2 * w + 1];
+          }
+          a.gate[t] = cn > 0.f ? sm / cn : 0.f;
+        }
+      }
     }
-    __syncthreads();
   }
   umma::fence_before_sync();
-  __syncthreads();
+  const bool failed = __syncthreads_or(!ok) != 0;  // the same decision on every thread
   if (a.amax)
     for (int i = tid; i < 6 * 32; i += kNetThreads) atomicMax(&a.amax[i], s_amax[i]);
   if (failed) {
-    // MMA batches may still be in flight: give each barrier a bounded chance to
-    // complete before the accumulator columns are released
-    for (int mt = 0; mt < kMaxMT; ++mt) umma::mbar_wait(mbar + mt, (phases >> mt) & 1u, 1u << 18);
+    if (tid == 0) atomicOr(a.status, kStTimeout);
+    // MMA batches may still be in flight: one more barrier behind them, with a
+    // bounded wait, before the accumulator columns are released
+    if (wid == kNetWorkers / 32 && umma::elect()) umma::mma_commit(drained);
+    umma::mbar_wait(drained, 0u, 1u << 18);
+    __syncthreads();
   }
   if (wid == 0) umma::tmem_dealloc(taddr, kTmemCols);
 }
@@ -776,10 +849,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
 //     and are never used), B = x moved by dy rows, 16 positions per MMA: three tap
 //     rows make nine taps. D (3 x 32 columns) stays in tensor memory over the CTA's
 //     tiles and goes to its partial sums at the end.
-// Lane 0 of warp mt issues the input gradient's M tile mt, warp kMaxMT's the weight
-// gradient, each committing to a barrier of its own; every wait is bounded. x
-// arrives while the input gradient runs, and the next tile's dY is loaded into
-// registers beside the MMAs.
+// The last warp issues every MMA: the input gradient's M tiles, each committing to a
+// barrier of its own, then, once x has arrived, the weight gradient; the other warps
+// read the M tiles back meanwhile. The weight gradient's three MMAs on one A keep it in
+// the collector (26 cycles an MMA against 41, so nothing else may come between them).
+// The next tile's dY is loaded into registers beside the MMAs; the bias gradient is
+// summed from them. Every wait is bounded.
+// At 512 tiles a 32 -> 32 layer takes 38 us (a thread issuing the weight gradient
+// beside others: 51).
 template <int L>
 __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   extern __shared__ uint8_t s_raw[];
@@ -790,10 +867,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   uint8_t *wsm = bufX + 4 * kNPos * 16;
   float *s_part = (float *)(wsm + wbytesT(1));  // [8 warps][32]
   float *s_db = s_part + 8 * 32;                // [32] bias gradient over the CTA's tiles
-  uint64_t *mbar = (uint64_t *)(s_db + 32);     // input gradient per M tile, weight gradient
-  uint32_t *s_taddr = (uint32_t *)(mbar + kMaxMT + 1);
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  uint64_t *mbar = (uint64_t *)(s_db + 32);     // input gradient per M tile, weight gradient, x arrived
+  uint32_t *s_taddr = (uint32_t *)(mbar + kMaxMT + 2);
+  const int tid = threadIdx.x, lane = tid & 31, wid = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int wq = wid & 3, wg = wid >> 2;
+  const bool worker = wid < kBwdWorkers / 32;
   constexpr int ci_n = cin(l), co_n = cout(l);
   constexpr int NW = l == 0 ? 16 : 32;            // weight-gradient N: c_in padded to 16
   constexpr int nK = kchunks(l);
@@ -813,7 +891,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     uint4 *z = (uint4 *)smem;
     for (int i = tid; i < (int)kBufD / 16 + 4 * kNPos; i += kBwdThreads) z[i] = make_uint4(0, 0, 0, 0);
     if (tid < 32) s_db[tid] = 0.f;
-    if (tid <= kMaxMT) umma::mbar_init(mbar + tid, 1);
+    if (tid <= kMaxMT + 1) umma::mbar_init(mbar + tid, tid <= kMaxMT ? 1 : kBwdWorkers);
     if (wid == 0) {
       umma::tmem_alloc(s_taddr, kBwdTmemCols);
       umma::tmem_relinquish();
@@ -833,94 +911,122 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     for (int g = 0; g < gD; ++g)
 #pragma unroll
       for (int j = 0; j < kDRegs; ++j) {
-        const int q = tid + j * kBwdThreads;
+        const int q = tid + j * kBwdWorkers;
         dv[g][j] = q < nK * 16 ? __ldg(ds + g * kNPos + q) : make_uint4(0, 0, 0, 0);
       }
   };
-  if ((int)blockIdx.x < a.n) load_dy(blockIdx.x);
+  if (worker && (int)blockIdx.x < a.n) load_dy(blockIdx.x);
   for (int t = blockIdx.x; t < a.n && !failed; t += gridDim.x) {
-    // operands of this tile (the previous tile's MMAs have completed)
-    const uint4 *xs = a.acts + ((size_t)t * 6 + l) * 4 * kNPos;
+    bool ok = true;
+    if (worker) {  // operands of this tile (the previous tile's MMAs have completed)
+      const uint4 *xs = a.acts + ((size_t)t * 6 + l) * 4 * kNPos;
 #pragma unroll
-    for (int g = 0; g < gX; ++g)
-      for (int q = tid; q < nX; q += kBwdThreads) cp_async16(sX + (uint32_t)((g * kNPos + q) * 16), xs + g * kNPos + q);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+      for (int g = 0; g < gX; ++g)
+        for (int q = tid; q < nX; q += kBwdWorkers)
+          cp_async16(sX + (uint32_t)((g * kNPos + q) * 16), xs + g * kNPos + q);
+      asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll
-    for (int g = 0; g < gD; ++g)
+      for (int g = 0; g < gD; ++g)
 #pragma unroll
-      for (int j = 0; j < kDRegs; ++j) {
-        const int q = tid + j * kBwdThreads;
-        if (q < nK * 16) {
+        for (int j = 0; j < kDRegs; ++j) {
+          const int q = tid + j * kBwdWorkers;
+          if (q < nK * 16) {
 #pragma unroll
-          for (int s = 0; s < 3; ++s) ((uint4 *)bufD)[(s * 4 + g) * kDPlane + kDPad + s + q] = dv[g][j];
-        }
-      }
-    if (l > 0) {  // the input gradient needs dY only
-      umma::fence_proxy_async();
-      umma::fence_before_sync();
-      __syncthreads();
-      umma::fence_after_sync();
-      if (lane == 0 && wid < MT) {  // M tile wid: 9 taps x kg / 2 MMAs
-        constexpr uint32_t idesc = umma::idesc_bf16(128, 32);
-        const uint64_t b0 = umma::desc(sW, 4 * 128, 128);
-        const uint64_t a0 = umma::desc(sD + (uint32_t)(wid * 128 * 16), kDPlane * 16, 128);
-        const uint32_t d = taddr + kColG + (uint32_t)(wid * 32);
-#pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const int shift = (tap / 3) * kGW + (tap % 3);
-#pragma unroll
-          for (int kp = 0; kp < kg / 2; ++kp) {
-            const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kDPlane + shift) * 16));
-            const uint64_t bd = umma::desc_add(b0, (uint32_t)((tap * kg + 2 * kp) * 4 * 128));
-            umma::mma_bf16(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
+            for (int s = 0; s < 3; ++s) ((uint4 *)bufD)[(s * 4 + g) * kDPlane + kDPad + s + q] = dv[g][j];
           }
         }
-        umma::mma_commit(mbar + wid);
-      }
-      __syncwarp();
+      umma::fence_proxy_async();
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    umma::fence_proxy_async();
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
-    if (lane == 0 && wid == kMaxMT) {  // weight gradient: 3 tap rows x nK MMAs
-      constexpr uint32_t idesc = umma::idesc_bf16(128, NW) | (1u << 15) | (1u << 16);  // A and B MN-major
-      const uint64_t a0 = umma::desc(sD + (uint32_t)(kDPad * 16), 128, kDPlane * 16);
-      const uint64_t b0 = umma::desc(sX, 128, kNPos * 16);
-#pragma unroll 2
-      for (int kc = 0; kc < nK; ++kc)
+    if (!worker) {
+      if (l > 0 && umma::elect()) {  // the input gradient needs dY only: per M tile 9 taps x kg / 2 MMAs
+        constexpr uint32_t idesc = umma::idesc_bf16(128, 32);
+        const uint64_t b0 = umma::desc(sW, 4 * 128, 128);
+        const uint64_t a00 = umma::desc(sD, kDPlane * 16, 128);
+#pragma unroll 1
+        for (int mt = 0; mt < MT; ++mt) {
+          const uint64_t a0 = umma::desc_add(a00, (uint32_t)(mt * 128 * 16));
+          const uint32_t d = taddr + kColG + (uint32_t)(mt * 32);
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
-          umma::mma_bf16(taddr + (uint32_t)(r * NW), umma::desc_add(a0, (uint32_t)(kc * 256)),
-                         umma::desc_add(b0, (uint32_t)((kc * 16 + r * kGW) * 16)), idesc, (any || kc > 0) ? 1u : 0u);
-      umma::mma_commit(mbar + kMaxMT);
-    }
-    __syncwarp();
-    any = true;
-    if (t + (int)gridDim.x < a.n) load_dy(t + (int)gridDim.x);
-    // bias gradient: sum of dY over the output window (fixed order per tile)
-    {
-      const int co = lane;
-      float sum = 0.f;
-      if (co < co_n) {
-        const uint16_t *col = (const uint16_t *)(bufD + (co >> 3) * kDPlane * 16) + (co & 7);
-#pragma unroll 8
-        for (int q = wid; q < vout * kGW; q += 8) sum += __uint_as_float((uint32_t)col[(kDPad + q) * 8] << 16);
+          for (int tap = 0; tap < 9; ++tap) {
+            const int shift = (tap / 3) * kGW + (tap % 3);
+#pragma unroll
+            for (int kp = 0; kp < kg / 2; ++kp) {
+              const uint64_t ad = umma::desc_add(a0, (uint32_t)(((2 * kp) * kDPlane + shift) * 16));
+              const uint64_t bd = umma::desc_add(b0, (uint32_t)((tap * kg + 2 * kp) * 4 * 128));
+              umma::mma_bf16(d, ad, bd, idesc, (tap | kp) != 0 ? 1u : 0u);
+            }
+          }
+          umma::mma_commit(mbar + mt);
+        }
       }
-      s_part[wid * 32 + co] = sum;
-    }
-    __syncthreads();
-    if (tid < 32) {
-      float sum = 0.f;
+      __syncwarp();
+      ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + kMaxMT + 1, ph));
+      umma::fence_after_sync();
+      if (ok && umma::elect()) {  // weight gradient: 3 tap rows x nK MMAs
+        constexpr uint32_t idesc = umma::idesc_bf16(128, NW) | (1u << 15) | (1u << 16);  // A and B MN-major
+        const uint64_t a0 = umma::desc(sD + (uint32_t)(kDPad * 16), 128, kDPlane * 16);
+        const uint64_t b0 = umma::desc(sX, 128, kNPos * 16);
+        auto step = [&](int kc, uint32_t acc) {
+          const uint64_t ad = umma::desc_add(a0, (uint32_t)(kc * 256)), bd = umma::desc_add(b0, (uint32_t)(kc * 256));
+          umma::mma_bf16_keep_a<umma::Collect::fill>(taddr, ad, bd, idesc, acc);
+          umma::mma_bf16_keep_a<umma::Collect::use>(taddr + NW, ad, umma::desc_add(bd, kGW * 16), idesc, acc);
+          umma::mma_bf16_keep_a<umma::Collect::lastuse>(taddr + 2 * NW, ad, umma::desc_add(bd, 2 * kGW * 16), idesc,
+                                                        acc);
+        };
+        step(0, any ? 1u : 0u);
+#pragma unroll 4
+        for (int kc = 1; kc < nK; ++kc) step(kc, 1u);
+        umma::mma_commit(mbar + kMaxMT);
+      }
+      __syncwarp();
+    } else {
+      // bias gradient: sum of dY over its window (zero outside), from the staged registers;
+      // the warp's sums are split over its lanes by halves, lane co ends with channel co
+      {
+        float v[32];
 #pragma unroll
-      for (int w = 0; w < 8; ++w) sum += s_part[w * 32 + tid];
-      s_db[tid] += sum;
+        for (int c = 0; c < 32; ++c) v[c] = 0.f;
+#pragma unroll
+        for (int g = 0; g < gD; ++g)
+#pragma unroll
+          for (int j = 0; j < kDRegs; ++j) {
+            const uint32_t w[4] = {dv[g][j].x, dv[g][j].y, dv[g][j].z, dv[g][j].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              v[g * 8 + 2 * k] += bf16_lo(w[k]);
+              v[g * 8 + 2 * k + 1] += bf16_hi(w[k]);
+            }
+          }
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) {
+          const bool up = (lane & h) != 0;
+#pragma unroll
+          for (int c = 0; c < h; ++c) {
+            const float keep = up ? v[c + h] : v[c], give = up ? v[c] : v[c + h];
+            v[c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+          }
+        }
+        s_part[wid * 32 + lane] = v[0];
+      }
+      if (t + (int)gridDim.x < a.n) load_dy(t + (int)gridDim.x);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      umma::fence_proxy_async();
+      umma::mbar_arrive(mbar + kMaxMT + 1);
+      asm volatile("bar.sync 1, %0;" ::"n"(kBwdWorkers) : "memory");  // s_part, and x for the ReLU derivative
+      if (tid < 32) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) sum += s_part[w * 32 + tid];
+        s_db[tid] += sum;
+      }
     }
-    bool ok = true;
-    if (l > 0) {
+    any = true;
+    if (l > 0 && worker) {
       uint4 *dout = a.dyo + (size_t)t * 4 * kNPos;
-      for (int mt = wg; mt < MT && ok; mt += 2) {
+      for (int mt = wg; mt < MT; mt += 2) {
         ok = __all_sync(0xffffffffu, umma::mbar_wait(mbar + mt, ph));
         if (!ok) break;
         umma::fence_after_sync();

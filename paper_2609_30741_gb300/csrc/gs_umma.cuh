@@ -92,6 +92,30 @@ __device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t a_desc, uint6
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// The same on an A that stays in the collector over consecutive MMAs of one thread: `fill` loads
+// it, `use` and `lastuse` read it again.
+enum class Collect { fill, use, lastuse };
+template <Collect C>
+__device__ __forceinline__ void mma_bf16_keep_a(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                               uint32_t accumulate) {
+#define GS_MMA_KEEP_A(mode)                                                                             \
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"                                       \
+               "tcgen05.mma.cta_group::1.kind::f16.collector::a::" mode " [%0], %1, %2, %3, p;\n\t}\n" \
+               ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)                      \
+               : "memory")
+  if (C == Collect::fill) GS_MMA_KEEP_A("fill");
+  else if (C == Collect::use) GS_MMA_KEEP_A("use");
+  else GS_MMA_KEEP_A("lastuse");
+#undef GS_MMA_KEEP_A
+}
+// True on one lane of a converged warp. MMAs issued behind it cost 41 cycles each at M = 128,
+// N = 32, K = 16 (the tensor core's own rate); behind a test of the thread index the compiler
+// cannot know that one lane is active, and they cost 99 to 123.
+__device__ __forceinline__ bool elect() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0u;
+}
 // arrive on the mbarrier once every MMA issued so far by this thread is complete
 __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -102,6 +126,9 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
 // ---- mbarrier ----
 __device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *mbar, uint32_t phase) {
   uint32_t ok;
