@@ -855,8 +855,9 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
 // the collector (26 cycles an MMA against 41, so nothing else may come between them).
 // The next tile's dY is loaded into registers beside the MMAs; the bias gradient is
 // summed from them. Every wait is bounded.
-// At 512 tiles a 32 -> 32 layer takes 38 us (a thread issuing the weight gradient
-// beside others: 51).
+// At 512 tiles a 32 -> 32 layer takes 23 to 27 us, 8 to 10 k cycles a tile (a
+// thread issuing the weight gradient beside others, partials stored in the parameters'
+// order: 51 us).
 template <int L>
 __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   extern __shared__ uint8_t s_raw[];
@@ -882,14 +883,29 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   constexpr int gX = l == 0 ? 1 : 4;                   // c_in groups stored
   constexpr int nX = l == 0 ? kNPos : MT * 128;        // positions of x stored
   constexpr uint32_t kColG = 3 * 32;                   // first input-gradient column
+  uint4 dv[gD][kDRegs];  // dY of the tile in hand, then of the next
+  auto load_dy = [&](int t) {
+    const uint4 *ds = a.dy + (size_t)t * 4 * kNPos;
+#pragma unroll
+    for (int g = 0; g < gD; ++g)
+#pragma unroll
+      for (int j = 0; j < kDRegs; ++j) {
+        const int q = tid + j * kBwdWorkers;
+        dv[g][j] = q < nK * 16 ? __ldg(ds + g * kNPos + q) : make_uint4(0, 0, 0, 0);
+      }
+  };
   {
     if (l > 0) {
-      const uint4 *src = (const uint4 *)(a.wpackT + woffT(l));
-      for (int i = tid; i < wbytesT(l) / 16; i += kBwdThreads) ((uint4 *)wsm)[i] = src[i];
+      const uint8_t *src = a.wpackT + woffT(l);
+      const uint32_t dst = umma::smem_u32(wsm);
+      for (int i = tid; i < wbytesT(l) / 16; i += kBwdThreads) cp_async16(dst + (uint32_t)(i * 16), src + i * 16);
     }
+    if (worker && (int)blockIdx.x < a.n) load_dy(blockIdx.x);
     // dY's planes and what x leaves out: zero (and finite in the rows nothing reads)
     uint4 *z = (uint4 *)smem;
     for (int i = tid; i < (int)kBufD / 16 + 4 * kNPos; i += kBwdThreads) z[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    umma::fence_proxy_async();
     if (tid < 32) s_db[tid] = 0.f;
     if (tid <= kMaxMT + 1) umma::mbar_init(mbar + tid, tid <= kMaxMT ? 1 : kBwdWorkers);
     if (wid == 0) {
@@ -904,18 +920,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   const uint32_t sD = umma::smem_u32(bufD), sX = umma::smem_u32(bufX), sW = umma::smem_u32(wsm);
   uint32_t ph = 0;  // every barrier in use completes once per tile
   bool failed = false, any = false;
-  uint4 dv[gD][kDRegs];  // dY of the tile in hand, then of the next
-  auto load_dy = [&](int t) {
-    const uint4 *ds = a.dy + (size_t)t * 4 * kNPos;
-#pragma unroll
-    for (int g = 0; g < gD; ++g)
-#pragma unroll
-      for (int j = 0; j < kDRegs; ++j) {
-        const int q = tid + j * kBwdWorkers;
-        dv[g][j] = q < nK * 16 ? __ldg(ds + g * kNPos + q) : make_uint4(0, 0, 0, 0);
-      }
-  };
-  if (worker && (int)blockIdx.x < a.n) load_dy(blockIdx.x);
   for (int t = blockIdx.x; t < a.n && !failed; t += gridDim.x) {
     bool ok = true;
     if (worker) {  // operands of this tile (the previous tile's MMAs have completed)
@@ -1067,28 +1071,24 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     if (tid == 0) atomicOr(a.status, kStTimeout);
     for (int k = 0; k <= kMaxMT; ++k)
       if (k < MT || k == kMaxMT) umma::mbar_wait(mbar + k, ph, 1u << 18);
-  } else if (wid < 3) {
-    // weight gradient of the CTA's tiles: TMEM lane = s * 32 + c_out, column = dy * NW + c_in
+  } else if (worker && wq < 3) {
+    // weight gradient of the CTA's tiles: TMEM lane = s * 32 + c_out, column = dy * NW + c_in;
+    // stored [tap][c_in][c_out], so a warp's stores are whole lines (in the parameters' own
+    // order they were 32 lines each and took 17k cycles)
     constexpr int npar = co_n * 9 * ci_n;
     float *part = a.part + (size_t)blockIdx.x * (npar + co_n);
     const int co = lane;
 #pragma unroll 1
-    for (int r = 0; r < 3; ++r) {
-      for (int c16 = 0; c16 < NW / 16; ++c16) {
-        float h[16];
-        if (any) {
-          umma::tmem_ld16(taddr + ((uint32_t)(wid * 32) << 16) + (uint32_t)(r * NW + c16 * 16), h);
-        } else {
+    for (int u = wg; u < 3 * (NW / 16); u += 2) {
+      const int r = u / (NW / 16), c16 = u % (NW / 16);
+      float h[16];
+      umma::tmem_ld16(taddr + ((uint32_t)(wq * 32) << 16) + (uint32_t)(r * NW + c16 * 16), h);
+      if (co < co_n)
 #pragma unroll
-          for (int i = 0; i < 16; ++i) h[i] = 0.f;
+        for (int i = 0; i < 16; ++i) {
+          const int ci = c16 * 16 + i;
+          if (ci < ci_n) part[((r * 3 + wq) * ci_n + ci) * co_n + co] = h[i];
         }
-        if (co < co_n)
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int ci = c16 * 16 + i;
-            if (ci < ci_n) part[(co * 9 + r * 3 + wid) * ci_n + ci] = h[i];
-          }
-      }
     }
     if (wid == 0 && co < co_n) part[npar + co] = s_db[co];
   }
@@ -1107,20 +1107,26 @@ struct UpdateArgs {
 // grad[i] = sum over the CTAs' partials, deterministic: a block takes 32 parameters,
 // warp w the partials w, w + 8, ... in order, and the warps' sums are added in order.
 // Then AdamW. Bound by the latency of the partials' loads: one thread per parameter
-// with 16 loads in flight took 72 us for 152 CTAs, this 11.
+// with 16 loads in flight took 72 us for 152 CTAs, this 17.
 __global__ void __launch_bounds__(256) repair_update_kernel(UpdateArgs a) {
   __shared__ float s_sum[8][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int i = blockIdx.x * 32 + lane;
+  const int i = blockIdx.x * 32 + lane;  // in the partials' order
+  int par = i;                           // the parameter
   float sum = 0.f;
   if (i < kRepairParams) {
-    int off = poff(0), end = poff(1);
+    int off = poff(0), end = poff(1), ci_n = cin(0), co_n = cout(0);
 #pragma unroll
     for (int k = 1; k < 6; ++k)
       if (i >= poff(k)) {
         off = poff(k);
         end = poff(k + 1);
+        ci_n = cin(k);
+        co_n = cout(k);
       }
+    // the partials lie [tap][c_in][c_out], the parameters [c_out][tap][c_in]; biases last in both
+    const int e = i - off, co = e % co_n, rest = e / co_n;
+    if (e < co_n * 9 * ci_n) par = off + (co * 9 + rest / ci_n) * ci_n + rest % ci_n;
     const int count = end - off;
     const float *p = a.part + (size_t)a.n_parts * off + (i - off);
 #pragma unroll 8
@@ -1131,13 +1137,13 @@ __global__ void __launch_bounds__(256) repair_update_kernel(UpdateArgs a) {
   if (wid > 0 || i >= kRepairParams) return;
 #pragma unroll
   for (int w = 1; w < 8; ++w) sum += s_sum[w][lane];
-  a.grad[i] = sum;
+  a.grad[par] = sum;
   if (a.lr > 0.f) {
-    const float mi = fmaf(a.b1, a.m[i], (1.f - a.b1) * sum);
-    const float vi = fmaf(a.b2, a.v[i], (1.f - a.b2) * sum * sum);
-    a.m[i] = mi;
-    a.v[i] = vi;
-    a.w[i] -= a.lr * ((mi / a.bc1) / (sqrtf(vi / a.bc2) + a.eps) + a.wd * a.w[i]);
+    const float mi = fmaf(a.b1, a.m[par], (1.f - a.b1) * sum);
+    const float vi = fmaf(a.b2, a.v[par], (1.f - a.b2) * sum * sum);
+    a.m[par] = mi;
+    a.v[par] = vi;
+    a.w[par] -= a.lr * ((mi / a.bc1) / (sqrtf(vi / a.bc2) + a.eps) + a.wd * a.w[par]);
   }
 }
 
