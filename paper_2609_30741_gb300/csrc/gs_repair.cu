@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(kPackThreads) repair_pack_kernel(const float *
                                                                    uint16_t *__restrict__ wpack,
                                                                    float *__restrict__ bias,
                                                                    uint16_t *__restrict__ wpackT) {
+  griddep_wait();
   if (blockIdx.x < kPackBlocks) pack_forward(blockIdx.x * kPackThreads + threadIdx.x, master, wpack, bias);
   else pack_backward((blockIdx.x - kPackBlocks) * kPackThreads + threadIdx.x, master, wpackT);
 }
@@ -710,6 +711,7 @@ struct TrainArgs {
 // labels; the warped pixels carry view-dependent colour the features cannot
 // see, so the label rates the fill alone)
 __global__ void __launch_bounds__(256) repair_stats_kernel(TrainArgs a) {
+  griddep_wait();
   const int t = blockIdx.x;
   const uint32_t te = a.tiles[t];
   const int frame = (int)(te >> 24), ty0 = (int)((te >> 12) & 0xfffu) * kRT, tx0 = (int)(te & 0xfffu) * kRT;
@@ -761,6 +763,7 @@ __global__ void __launch_bounds__(256) repair_stats_kernel(TrainArgs a) {
 // then a tree), so a training step's loss terms do not depend on scheduling.
 __global__ void __launch_bounds__(1024) repair_sums_kernel(const float *__restrict__ tile_stats, int n, int fa, int fb,
                                                            float *__restrict__ sums, int s0) {
+  griddep_wait();
   __shared__ float red[1024];
   for (int k = 0; k < 2; ++k) {
     const int f = k ? fb : fa;
@@ -783,6 +786,7 @@ __device__ __forceinline__ float psnr_of(float mse) { return mse > 0.f ? -10.f *
 // the BF16 operand of the backward: channel group 0 (the only one it reads) holds
 // the 4 outputs, zero outside the window
 __global__ void __launch_bounds__(256) repair_dout_kernel(TrainArgs a) {
+  griddep_wait();
   const int t = blockIdx.x;
   const uint32_t te = a.tiles[t];
   const int frame = (int)(te >> 24), ty0 = (int)((te >> 12) & 0xfffu) * kRT, tx0 = (int)(te & 0xfffu) * kRT;
@@ -900,18 +904,21 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
       const uint32_t dst = umma::smem_u32(wsm);
       for (int i = tid; i < wbytesT(l) / 16; i += kBwdThreads) cp_async16(dst + (uint32_t)(i * 16), src + i * 16);
     }
-    if (worker && (int)blockIdx.x < a.n) load_dy(blockIdx.x);
     // dY's planes and what x leaves out: zero (and finite in the rows nothing reads)
     uint4 *z = (uint4 *)smem;
     for (int i = tid; i < (int)kBufD / 16 + 4 * kNPos; i += kBwdThreads) z[i] = make_uint4(0, 0, 0, 0);
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    umma::fence_proxy_async();
     if (tid < 32) s_db[tid] = 0.f;
     if (tid <= kMaxMT + 1) umma::mbar_init(mbar + tid, tid <= kMaxMT ? 1 : kBwdWorkers);
     if (wid == 0) {
       umma::tmem_alloc(s_taddr, kBwdTmemCols);
       umma::tmem_relinquish();
     }
+    // the set-up above runs while the kernel before drains; the weights are older than that
+    // kernel, which itself waited for what came before it
+    griddep_wait();
+    if (worker && (int)blockIdx.x < a.n) load_dy(blockIdx.x);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    umma::fence_proxy_async();
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
@@ -1109,6 +1116,7 @@ struct UpdateArgs {
 // Then AdamW. Bound by the latency of the partials' loads: one thread per parameter
 // with 16 loads in flight took 72 us for 152 CTAs, this 17.
 __global__ void __launch_bounds__(256) repair_update_kernel(UpdateArgs a) {
+  griddep_wait();
   __shared__ float s_sum[8][32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;  // in the partials' order
@@ -1184,8 +1192,8 @@ cudaError_t prepare_repair() {
 }
 
 cudaError_t repair_pack(const Workspace &ws, cudaStream_t s) {
-  repair_pack_kernel<<<kPackBlocks + kPackTBlocks, kPackThreads, 0, s>>>(ws.rp_master, (uint16_t *)ws.rp_wpack,
-                                                                         ws.rp_bias, (uint16_t *)ws.rp_wpackT);
+  launch_k(repair_pack_kernel, kPackBlocks + kPackTBlocks, kPackThreads, 0, s, ws.rp_master, (uint16_t *)ws.rp_wpack,
+           ws.rp_bias, (uint16_t *)ws.rp_wpackT);
   GS_LAUNCHED(1);
   return cudaGetLastError();
 }
@@ -1308,10 +1316,10 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
   a.tile_stats = stats;
   a.sums = sums;
   a.lam = o.gate_weight;
-  repair_stats_kernel<<<n, 256, 0, s>>>(a);
-  repair_sums_kernel<<<1, 1024, 0, s>>>(stats, n, 2, 4, sums, 0);  // holes, L1 sum
-  repair_dout_kernel<<<n, 256, 0, s>>>(a);
-  repair_sums_kernel<<<1, 1024, 0, s>>>(stats, n, 5, 6, sums, 2);  // BCE, positive labels
+  launch_k(repair_stats_kernel, n, 256, 0, s, a);
+  launch_k(repair_sums_kernel, 1, 1024, 0, s, stats, n, 2, 4, sums, 0);  // holes, L1 sum
+  launch_k(repair_dout_kernel, n, 256, 0, s, a);
+  launch_k(repair_sums_kernel, 1, 1024, 0, s, stats, n, 5, 6, sums, 2);  // BCE, positive labels
   GS_LAUNCHED(4);
   // backward, last layer first: per layer one tensor-core kernel (weight
   // gradient into per-CTA partials, input gradient into the other buffer); the
@@ -1326,7 +1334,7 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
     ba.part = part + (size_t)G * poff(l);
     ba.n = n;
     ba.status = &ws.ctr->status;
-    bwd_kernel(l)<<<G, kBwdThreads, bwd_smem(), s>>>(ba);
+    launch_k(bwd_kernel(l), G, kBwdThreads, bwd_smem(), s, ba);
     GS_LAUNCHED(1);
     uint4 *tmp = cur;
     cur = nxt;
@@ -1346,7 +1354,7 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
   u.wd = o.weight_decay;
   u.bc1 = 1.f - powf(o.beta1, (float)o.step);
   u.bc2 = 1.f - powf(o.beta2, (float)o.step);
-  repair_update_kernel<<<(kRepairParams + 31) / 32, 256, 0, s>>>(u);
+  launch_k(repair_update_kernel, (kRepairParams + 31) / 32, 256, 0, s, u);
   GS_LAUNCHED(1);
   if (o.lr > 0.f)
     if ((e = repair_pack(ws, s)) != cudaSuccess) return e;
