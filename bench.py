@@ -702,7 +702,7 @@ def run_ours(args):
         "preprocess": hbm_line("preprocess_kernel (stage: the kernel alone, both eyes' records)",
                                PREPROCESS_BYTES_PER_SURFEL * scene.n, st_stereo[0],
                                f"{PREPROCESS_BYTES_PER_SURFEL} B x {scene.n} surfels"),
-        "binning_dominant": hbm_line("dominant-eye binning (compaction, row spans, depth sort, band lists, "
+        "binning_dominant": hbm_line("dominant-eye binning (row spans, depth sort, row lists, "
                                      "counting sort by tile)", BIN_BYTES_PER_INSTANCE * inst_dom, st_stereo[1],
                                      f"{BIN_BYTES_PER_INSTANCE} B x {inst_dom:.4g} instances"),
         "warp_classify": hbm_line("warp, edge ROIs, gap classification", WARP_BYTES_PER_PIXEL * W * H, st_stereo[3],
