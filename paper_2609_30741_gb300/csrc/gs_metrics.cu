@@ -4,9 +4,14 @@
 // C1 = 0.01^2, C2 = 0.03^2, the mean of the SSIM map over every pixel of every
 // channel.
 //
-// One CTA per 32 x 32 output tile and channel. The four filtered quantities x, y,
-// x^2 + y^2 and x y (the formula needs only the sum of the two second moments)
-// are kept as two FP32x2 pairs. The 42 x 42 window of both images (zero outside)
+// One CTA per 32 x 32 output tile and channel. Four quantities are filtered, as two
+// FP32x2 pairs: a = x + y and d = x - y, and their squares. With A, D their means and
+// va, vd their variances, 2 mx my = (A^2 - D^2) / 2, mx^2 + my^2 = (A^2 + D^2) / 2, and
+// likewise 2 sxy and sxx + syy from va and vd. For images that differ little (what a
+// quality metric is asked about) d is small and nearly exact, and the rounding of va,
+// which is that of squares near 4, enters numerator and denominator alike: flat white
+// with noise of 1e-4 is 1e-7 from the 64-bit value, and was 1e-5 from x^2 + y^2 and x y.
+// The 42 x 42 window of both images (zero outside)
 // goes to shared memory interleaved; a thread filters four columns of a row from
 // sixteen pixels in registers, and then eight rows of a column from eighteen
 // filtered rows, so an output costs four 16-byte shared-memory loads in place of
@@ -31,7 +36,7 @@ constexpr float kC1 = 0.01f * 0.01f, kC2 = 0.03f * 0.03f;
 
 constexpr int kSsThreads = 128;
 constexpr int kSsCtas = 5;                // resident CTAs per SM
-constexpr int kSsUnits = 24;             // 16-byte units (two pixels of both images) of a window row: 22, padded
+constexpr int kSsUnits = 24;             // 16-byte units (a and d of two pixels) of a window row: 22, padded
 constexpr int kSsCols = 4, kSsRows = 8;  // columns and rows a thread filters at a time
 
 struct GaussW {
@@ -57,7 +62,7 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
   // window rows: even units first, then odd ones, so the eight threads of a row
   // read consecutive units
   __shared__ float4 s_in[kSsW][kSsUnits];
-  __shared__ float4 s_h[kSsW][kSsT];  // horizontally filtered: x, y, x^2 + y^2, x y
+  __shared__ float4 s_h[kSsW][kSsT];  // horizontally filtered: a, d, a^2, d^2
   __shared__ double s_red[kSsThreads];
   __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -95,7 +100,8 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
     for (int h = 0; h < 2; ++h) {
       const int c = lane + 32 * h, u = c >> 1;
       if (c < 2 * 22)  // columns 42 and 43 pad the last unit
-        reinterpret_cast<float2 *>(&s_in[r][(u & 1) * 12 + (u >> 1)])[c & 1] = make_float2(va[i][h], vb[i][h]);
+        reinterpret_cast<float2 *>(&s_in[r][(u & 1) * 12 + (u >> 1)])[c & 1] =
+            make_float2(va[i][h] + vb[i][h], va[i][h] - vb[i][h]);
     }
   }
   __syncthreads();
@@ -110,14 +116,13 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
       const float4 q = s_in[r][(u & 1) * 12 + g + (u >> 1)];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float x = h ? q.z : q.x, y = h ? q.w : q.y;
-        const float2 xy = make_float2(x, y), qq = make_float2(fmaf(x, x, y * y), x * y);
+        const float2 ad = h ? make_float2(q.z, q.w) : make_float2(q.x, q.y), qq = __fmul2_rn(ad, ad);
 #pragma unroll
         for (int o = 0; o < kSsCols; ++o) {
           const int k = 2 * u + h - o;  // tap
           if (k < 0 || k > 2 * kSsR) continue;
           const float2 w = w2[k <= kSsR ? k : 2 * kSsR - k];
-          m[o] = __ffma2_rn(w, xy, m[o]);
+          m[o] = __ffma2_rn(w, ad, m[o]);
           v[o] = __ffma2_rn(w, qq, v[o]);
         }
       }
@@ -149,10 +154,9 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
 #pragma unroll
     for (int o = 0; o < kSsRows; ++o) {
       if (ty0 + r0 + o >= H || tx0 + c >= W) continue;
-      const float mx = m[o].x, my = m[o].y;
-      const float mm = fmaf(mx, mx, my * my), xy = mx * my;
-      const float ss = v[o].x - mm, sxy = v[o].y - xy;
-      add_to(sum, err, ((2.f * xy + kC1) * (2.f * sxy + kC2)) / ((mm + kC1) * (ss + kC2)));
+      const float2 mm = __fmul2_rn(m[o], m[o]), vv = __ffma2_rn(make_float2(-m[o].x, -m[o].y), m[o], v[o]);
+      add_to(sum, err, ((mm.x - mm.y + 2.f * kC1) * (vv.x - vv.y + 2.f * kC2)) /
+                           ((mm.x + mm.y + 2.f * kC1) * (vv.x + vv.y + 2.f * kC2)));
     }
   }
   }

@@ -1,0 +1,40 @@
+"""GPU SSIM (gs_ssim) of images that differ little, against the FP64 oracle.
+
+With d the images' difference the map is (1 - D^2 / (..)) (1 - vd / (..)): d^2 is at most
+1e-6 here, so the rounding of the filters (22 FP32 steps, 2^-19 relative) moves a map
+value by less than 1e-8, and what is left is the rounding of the map's own seven
+operations and of the result: 8 x 2^-24 in all.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 8 * 2.0 ** -24
+
+
+@pytest.fixture(scope="module")
+def gs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_30741_gb300 import build
+    build.build()
+    from paper_2609_30741_gb300 import gs as gsmod
+    return gsmod
+
+
+@pytest.mark.parametrize("noise", [1e-4, 1e-3])
+@pytest.mark.parametrize("kind", ["white", "bright", "grey"])
+@pytest.mark.parametrize("shape", [(3, 37, 53), (1, 240, 321)])
+def test_ssim_of_close_images(gs, shape, kind, noise):
+    from oracle import metrics
+    rng = np.random.default_rng(shape[1])
+    x = {"white": np.ones(shape), "bright": 0.9 + 0.1 * rng.random(shape), "grey": np.full(shape, 0.5)}[kind]
+    y = x + noise * np.clip(rng.standard_normal(shape), -3.0, 3.0)
+    a, b = (torch.tensor(v, dtype=torch.float32, device="cuda") for v in (x, y))
+    ctx = gs.Context(16, 512, 512, max_instances=1 << 12)
+    want = metrics.ssim(a.double().cpu().numpy(), b.double().cpu().numpy())
+    for p, q in ((a, b), (b, a)):
+        assert abs(float(ctx.ssim(p, q)) - want) <= TOL, (float(ctx.ssim(p, q)), want)
+    assert float(ctx.ssim(b, b)) == 1.0
