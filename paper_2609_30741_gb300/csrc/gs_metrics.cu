@@ -15,13 +15,13 @@
 // goes to shared memory interleaved; a thread filters four columns of a row from
 // sixteen pixels in registers, and then eight rows of a column from eighteen
 // filtered rows, so an output costs four 16-byte shared-memory loads in place of
-// 77 4-byte ones. The map's sum is carried as an unevaluated float pair (the
-// compensated sum is as exact as the double it replaces; FP64 runs at a fiftieth
-// of the FP32 rate here) over the tiles a CTA takes, written in double, and the
-// last CTA adds the partial sums in a fixed order, so the result does not depend
-// on scheduling.
-// 1919 x 1079 x 3: 59 us, bound by instruction issue (41M warp instructions); 84 + 6
-// us for 4-byte loads, five quantities, double sums and a kernel to add them.
+// 77 4-byte ones. The map's sum is a double. FP64 runs at a fiftieth of
+// the FP32 rate here, so a thread first adds its eight values of a tile as an
+// unevaluated float pair (exact for values from 2^-19 to 2, within 2^-40 of smaller
+// ones) and then the pair to the double. The last CTA adds the partial sums in
+// a fixed order, so the result does not depend on scheduling.
+// 1919 x 1079 x 3: 57 us a call, bound by instruction issue; 94 for 4-byte loads, five
+// quantities, a double addition per value and a kernel to add the sums.
 #include "gs_internal.cuh"
 #include "gs_launch.cuh"
 
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
   float2 w2[kSsR + 1];  // the weights are symmetric
 #pragma unroll
   for (int k = 0; k <= kSsR; ++k) w2[k] = make_float2(gw.w[k], gw.w[k]);
-  float sum = 0.f, err = 0.f;
+  double total = 0.0;
   if (blockIdx.x < n) load(blockIdx.x);
   for (uint32_t t = blockIdx.x; t < n; t += gridDim.x) {
 #pragma unroll
@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
         v[o] = __ffma2_rn(w, make_float2(q.z, q.w), v[o]);
       }
     }
+    float sum = 0.f, err = 0.f;
 #pragma unroll
     for (int o = 0; o < kSsRows; ++o) {
       if (ty0 + r0 + o >= H || tx0 + c >= W) continue;
@@ -158,15 +159,13 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
       add_to(sum, err, ((mm.x - mm.y + 2.f * kC1) * (vv.x - vv.y + 2.f * kC2)) /
                            ((mm.x + mm.y + 2.f * kC1) * (vv.x + vv.y + 2.f * kC2)));
     }
+    total += (double)sum;
+    if (isfinite(sum)) total += (double)err;  // of an infinite sum the error term is NaN
   }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float s2 = __shfl_xor_sync(0xffffffffu, sum, o), e2 = __shfl_xor_sync(0xffffffffu, err, o);
-    add_to(sum, err, s2);
-    err += e2;
-  }
-  if (lane == 0) s_red[warp] = isfinite(sum) ? (double)sum + (double)err : (double)sum;
+  for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+  if (lane == 0) s_red[warp] = total;
   __syncthreads();
   if (tid == 0) {
     part[blockIdx.x] = ((s_red[0] + s_red[1]) + s_red[2]) + s_red[3];
