@@ -13,8 +13,10 @@ namespace gs {
 
 // Do all samples keep their row? Rrel, trel: dominant camera -> affiliated camera.
 // With Y / Z = (d (r_y + e1) + t1) / (d (1 + e2) + t2), Z > kZNear, the projected
-// row differs from the source's by at most fy times the bound below; a quarter of
-// a pixel leaves room for the float32 evaluation (2^-22 of 8192 rows is 0.002).
+// row differs from the source's by at most fy times the bound below, for which a
+// quarter of a pixel is allowed. The other quarter is for the float32 evaluation: six
+// roundings of y - cy and two of the row, below 2^-21 (H + |cy|) in all (0.006 pixel at
+// 8192 rows; past 2^19 rows, or with the principal point as far off, the scatter).
 inline bool rows_kept(const double *Rrel, const double *trel, double fx, double fy, double cx, double cy, int W,
                       int H) {
   const double rx = fmax(fabs(cx), fabs(W - 1.0 - cx)) / fx, ry = fmax(fabs(cy), fabs(H - 1.0 - cy)) / fy;
@@ -23,7 +25,7 @@ inline bool rows_kept(const double *Rrel, const double *trel, double fx, double 
   const double t1 = fabs(trel[1]), t2 = fabs(trel[2]), z = (double)kZNear;
   if (!(e2 < 0.5)) return false;
   const double off = (e1 + ry * e2) * (1.0 + t2 / z) / (1.0 - e2) + (t1 + ry * t2) / z;
-  return fy * off < 0.25;
+  return fy * off < 0.25 && 0x1p-21 * (H + fabs(cy)) < 0.25;
 }
 
 // The relative pose X_a = Rrel X_d + trel in FP64 (Eq. 4 followed by Eq. 5), each
