@@ -340,6 +340,7 @@ __device__ __forceinline__ void raster_items(const RasterTable &tab, uint32_t *q
       __syncwarp();
       if (nq & 1) {
         if (lane < 17) wq[2 * lane] = qp[2 * lane];
+        __syncwarp();  // the odd record has left its slot before a lane fills it again
       }
       nq &= 1;
     };
