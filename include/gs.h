@@ -169,8 +169,10 @@ typedef struct {
 
 /* Work counts of a context's last call, for sizing a context to a workload:
  * per eye the binned surfels, the (surfel, tile) instances, the (surfel, tile
- * row) spans and the (surfel, band of 4 tile rows) list entries the binning
- * produced (counted also when they overflowed a capacity). */
+ * row) spans and the (surfel, band of 4 tile rows) pairs the binning produced
+ * (counted also when they overflowed a capacity). An instance capacity of at
+ * least the instances and the spans holds the frame; no buffer is sized by the
+ * pairs. */
 typedef struct {
   int64_t binned[2], instances[2], spans[2], band_entries[2];
 } gs_usage;

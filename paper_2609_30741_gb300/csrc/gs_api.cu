@@ -76,7 +76,6 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   for (int e = 0; e < 2; ++e) {
     const size_t bytes = 12 * (Ie[e] < few ? Ie[e] : few) + pool_more;
     ws.row_pool_cap[e] = (uint32_t)(bytes / kRowEntryBytes + 1024);
-    ws.band_cap[e] = (uint32_t)(Ie[e] < 8 * N ? Ie[e] + 1024 : 8 * N + 1024);
   }
   const size_t rs_words = radix_status_words(N);
   for (int e = 0; e < 2; ++e) {  // one binning scratch per eye

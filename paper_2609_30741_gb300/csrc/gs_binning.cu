@@ -403,7 +403,8 @@ struct ReuseApply {
 //     counts of the warps before it and writes every surfel id to its slot.
 constexpr int kBinWarps = 8;
 constexpr int kBinThreads = kBinWarps * 32;
-constexpr int kBandRows = 4;    // rows of a band (gs_usage counts (surfel, band) pairs)
+constexpr int kBandRows = 4;    // rows of a band (gs_usage counts (surfel, band) pairs with a row entry)
+static_assert(kBandRows == 4, "row_list_kernel finds a band's rows in a block's nibbles");
 constexpr int kCountRows = 4;   // rows a counting CTA takes
 
 // One (surfel, row range): surfel id, first column | last column << 16.
@@ -419,15 +420,13 @@ struct ListArgs {
   const uint4 *info;       // per surfel: rectangle, slot of its first row in spans, flags (rows_kernel)
   const uint2 *spans;      // tile ranges of every rectangle row (rows_kernel)
   uint32_t span_cap;
-  const uint32_t *sat;     // ROI mask summed-area table, or null
-  const uint16_t *clip;    // per row and column the next masked column, or null
+  const uint16_t *clip;    // ROI mask: per row and column the next masked column, or null
   int tiles_x, tiles_y;
   uint32_t warp_surfels;
   RowEntry *pool;          // all lists
   uint32_t pool_cap;
   uint32_t *pool_n;        // entries taken (device counter)
-  uint32_t *n_band;        // (surfel, band) pairs (device counter), and their bound
-  uint32_t band_cap;
+  uint32_t *n_band;        // (surfel, band) pairs (device counter)
   uint2 *lists;            // [chunk][row][warp]: (first entry, entries)
   uint32_t *status;
 };
@@ -529,8 +528,7 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
         uint32_t base = 0;
         if (run > 0) base = atomicAdd(a.pool_n, run);
         if (run > 0 && (uint64_t)base + run > a.pool_cap) atomicOr(a.status, kStCapacity);
-        if (s_bands > 0 && (uint64_t)atomicAdd(a.n_band, s_bands) + s_bands > a.band_cap)
-          atomicOr(a.status, kStCapacity);
+        if (s_bands > 0) atomicAdd(a.n_band, s_bands);
         s_base = base;
       }
       __syncthreads();
@@ -560,14 +558,6 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
         x1 = (int)(inf.y & 0xffffu); y1 = (int)(inf.y >> 16);
         ro = inf.z;
         split = (inf.w & kInfoSplit) != 0u;
-        if (pass == 0) {
-          const int b0 = y0 / kBandRows, b1 = y1 / kBandRows;
-          if (!a.clip) bands += (uint32_t)(b1 - b0 + 1);
-          else
-            for (int b = b0; b <= b1; ++b)
-              bands += sat_any(a.sat, a.tiles_x, max(y0, b * kBandRows), min(y1, b * kBandRows + kBandRows - 1), x0,
-                               x1);
-        }
       }
       const bool any_split = __any_sync(0xffffffffu, split);
       const bool has = y0 <= y1;
@@ -603,6 +593,9 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
           cb = transpose_bits(rb, lane);
         }
         if (pass == 0) {
+          uint32_t any4 = ra | (ra >> 1);
+          any4 |= any4 >> 2;  // bit 4 b: a row of the block's band b
+          bands += (uint32_t)__popc(any4 & 0x11111111u);
           if (base + lane < ny) cnt[base + lane] += (uint32_t)(__popc(ca) + __popc(cb));
         } else {
           col[blk * 32 + lane] = ca;
@@ -963,7 +956,6 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   la.info = ws.info[eye];
   la.spans = ws.spans[eye];
   la.span_cap = cap;
-  la.sat = tile_mask ? b.mask_sat : nullptr;
   la.clip = tile_mask ? b.mask_clip : nullptr;
   la.tiles_x = tiles_x;
   la.tiles_y = tiles_y;
@@ -972,7 +964,6 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   la.pool_cap = ws.row_pool_cap[eye];
   la.pool_n = &ctr->n_entries[eye];
   la.n_band = &ctr->n_band[eye];
-  la.band_cap = ws.band_cap[eye];
   la.lists = b.row_lists;
   la.status = &ctr->status;
   launch_k(row_list_kernel, ws.bin_nch * kBinWarps, kBinThreads, list_smem_bytes(tiles_y), s, la);

@@ -130,7 +130,6 @@ struct Workspace {
   uint32_t *vis[2];             // one bit per surfel and eye: its rectangle is not empty
   uint32_t *cnt_bin;            // tiles each surfel reaches in the last binning (keep_intermediates)
   uint32_t row_pool_cap[2];     // entries of row_pool, per eye
-  uint32_t band_cap[2];         // bound on an eye's (surfel, band of 4 tile rows) pairs
   BinScratch bin[2];            // per eye
   uint8_t *tile_mask;           // ROI mask on the 16-pixel grid
   uint8_t *strip_mask;          // edge-strip tiles of a reused depth range (16-pixel grid)

@@ -316,7 +316,7 @@ class Context:
         _check(lib().gs_context_set_stream(self.h, C.c_void_p(stream.cuda_stream)), "gs_context_set_stream")
 
     def usage(self):
-        """Per-eye binned surfels, instances, spans and band-list entries of the
+        """Per-eye binned surfels, instances, spans and (surfel, band) pairs of the
         last call (synchronises the context's stream)."""
         u = Usage()
         _check(lib().gs_context_usage(self.h, C.byref(u)), "gs_context_usage")
