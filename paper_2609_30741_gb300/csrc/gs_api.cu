@@ -66,16 +66,13 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   ws.bin_nch = bin_chunks(lim.max_surfels);
   const size_t table = tiles * ws.bin_nch;
   ws.cnt_bin = c.take<uint32_t>(lim.keep_intermediates ? N : 1);
-  // the row-list entries are the spans, but for an ROI binning's rows without a
-  // masked tile, and one more for each of the few spans with two ranges: an eighth
-  // more entries than spans hold them (9 B per span). 12 B for each of the first 8
-  // spans per surfel cover that; for capacities far beyond, both eyes' pools get
-  // what the larger one still needs.
-  const size_t few = 8 * N, most = Ie[0] > Ie[1] ? Ie[0] : Ie[1];
-  const size_t pool_more = 9 * most > 12 * few ? 9 * most - 12 * few : 0;
+  // a row list holds an entry for each of the eye's spans (but for an ROI binning's
+  // rows without a masked tile) and one for each second range. A surfel's low-pass
+  // disc is at most 4.8 pixels high and lies in two tile rows, so it has two second
+  // ranges at most: with 8 per surfel a frame whose spans fit always fits.
   for (int e = 0; e < 2; ++e) {
-    const size_t bytes = 12 * (Ie[e] < few ? Ie[e] : few) + pool_more;
-    ws.row_pool_cap[e] = (uint32_t)(bytes / kRowEntryBytes + 1024);
+    ws.more_cap[e] = (uint32_t)(Ie[e] < 8 * N ? Ie[e] : 8 * N);
+    ws.row_pool_cap[e] = (uint32_t)Ie[e] + ws.more_cap[e];
   }
   const size_t rs_words = radix_status_words(N);
   for (int e = 0; e < 2; ++e) {  // one binning scratch per eye
@@ -88,7 +85,7 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
     b.ival = c.take<uint32_t>(Ie[e]);
     b.ikey = c.take<uint32_t>(lim.keep_intermediates ? Ie[e] : 1);
     b.bin_table = c.take<uint4>(table);
-    b.row_pool = reinterpret_cast<RowEntry *>(c.take<char>(kRowEntryBytes * ws.row_pool_cap[e]));
+    b.row_pool = c.take<uint32_t>(ws.row_pool_cap[e]);
     b.row_lists = c.take<uint2>(row_list_words(lim.max_surfels, (int)rty));  // the binning runs on the raster grid
     b.bin_offs = c.take<uint32_t>(table);
     b.ranges = c.take<uint2>(tiles);
@@ -112,7 +109,8 @@ void layout(const gs_limits &lim, Carver &c, Workspace &ws) {
   ws.strip_rgb = c.take<float>(reuse ? 3 * P : 1);
   for (int e = 0; e < 2; ++e) {
     ws.info[e] = c.take<uint4>(N);
-    ws.spans[e] = c.take<uint2>(Ie[e]);
+    ws.spans[e] = c.take<uint32_t>(Ie[e]);
+    ws.more[e] = c.take<uint2>(ws.more_cap[e]);
   }
   ws.warpbuf = c.take<unsigned long long>(stereo ? P : 1);
   ws.warp_depth = c.take<float>(stereo ? P : 1);

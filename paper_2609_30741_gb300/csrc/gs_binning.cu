@@ -96,9 +96,10 @@ __global__ void __launch_bounds__(1024) mask_sat_kernel(uint8_t *mask, int tiles
                                                         uint32_t *__restrict__ sat, const uint8_t *__restrict__ roi16,
                                                         int rtx, int rty, int tshift, uint16_t *__restrict__ clip,
                                                         uint32_t *__restrict__ list16,
-                                                        uint32_t *__restrict__ n_rows) {
+                                                        uint32_t *__restrict__ n_rows,
+                                                        uint32_t *__restrict__ n_more) {
   griddep_wait();
-  if (threadIdx.x == 0) *n_rows = 0u;  // the row spans of this binning follow
+  if (threadIdx.x == 0) *n_rows = *n_more = 0u;  // the row spans of this binning follow
   constexpr int kSatSmem = 12000;
   __shared__ uint32_t s_sat[kSatSmem];
   __shared__ uint32_t s_n16;
@@ -215,17 +216,27 @@ __device__ __forceinline__ void clip_to_mask(const uint16_t *clip, int tiles_x, 
 }
 
 // ---------------------------------------------------------------- row spans
-// Flags of a surfel's info: binned by this eye; has a row with two ranges.
-constexpr uint32_t kInfoBinned = 1u, kInfoSplit = 2u;
+constexpr uint32_t kInfoBinned = 1u;  // of a surfel's info: binned by this eye
+// A range of tile columns [lo, hi] (empty: [1, 0]) in 18 bits.
+constexpr int kColBits = 9;
+constexpr uint32_t kColMask = (1u << kColBits) - 1u, kNoRange = 1u << kColBits;
+static_assert(kMaxTileCols <= 1 << kColBits, "tile columns of a range");
+__device__ __forceinline__ uint32_t pack_range(int lo, int hi) { return (uint32_t)lo << kColBits | (uint32_t)hi; }
+__device__ __forceinline__ int range_lo(uint32_t r) { return (int)(r >> kColBits & kColMask); }
+__device__ __forceinline__ int range_hi(uint32_t r) { return (int)(r & kColMask); }
 
 // Once per eye and frame, every tile row of every surfel's bounding rectangle
-// gets its tile ranges [a0, a1] u [c0, c1] (row_ranges; an ill-conditioned
-// ellipse keeps the whole row of its rectangle), packed as 4 x 16 bits. A warp
+// gets its tile range [a0, a1] (row_ranges; an ill-conditioned ellipse keeps the
+// whole row of its rectangle), packed as 2 x 9 bits. The few rows with a second
+// range (the low-pass disc apart from the ellipse: at most two a surfel) put it in
+// `more`, a surfel's chained from its info. Half the bytes of two ranges a row, and
+// the row lists gather them at random. A warp
 // takes 32 consecutive surfels (one per lane), reserves slots for all their rows
 // with one atomic, and then computes the rows 32 at a time, one per lane, so no
 // lane idles while another walks a large surfel. info[i] collects what the row
 // lists need of surfel i in one 16-byte record, because they gather it at random
-// in depth order: the rectangle, the slot of its first row and flags. An ROI
+// in depth order: the rectangle, the slot of its first row, and above the flag that
+// this eye bins it the place of its first second range in `more`, plus one. An ROI
 // binning keeps of each range only the part from its first to its last masked
 // tile, skips the surfels whose rectangle holds no ROI tile, and marks the others
 // in `bits`, the selection its depth order is taken from: the test then runs once
@@ -235,9 +246,10 @@ __global__ void __launch_bounds__(256) rows_kernel(uint32_t n, const float4 *__r
                                                    const ushort4 *__restrict__ rect,
                                                    const uint32_t *__restrict__ vis,
                                                    const CamBlock *__restrict__ cams, int eye, int prim,
-                                                   uint4 *__restrict__ info, uint2 *__restrict__ spans,
+                                                   uint4 *__restrict__ info, uint32_t *__restrict__ spans,
                                                    uint32_t cap, uint32_t *__restrict__ n_rows,
-                                                   uint32_t *__restrict__ status, const uint16_t *__restrict__ clip,
+                                                   uint2 *__restrict__ more, uint32_t more_cap,
+                                                   uint32_t *__restrict__ n_more, uint32_t *__restrict__ status, const uint16_t *__restrict__ clip,
                                                    int clip_tiles_x, int clip_tiles_y,
                                                    const uint32_t *__restrict__ sat, uint32_t *__restrict__ bits) {
   griddep_wait();
@@ -283,7 +295,7 @@ __global__ void __launch_bounds__(256) rows_kernel(uint32_t n, const float4 *__r
   if (lane == 31 && total > 0) base = atomicAdd(n_rows, (uint32_t)total);
   base = __shfl_sync(0xffffffffu, base, 31);
   if (lane == 0 && total > 0 && (uint64_t)base + (uint64_t)total > cap) atomicOr(status, kStCapacity);
-  uint32_t split = 0;  // bit k: surfel k of the warp has a row with two ranges
+  uint32_t head = 0;  // the surfel's second ranges: place in `more` plus one, or none
   for (int q0 = 0; q0 < total; q0 += 32) {
     const int qq = q0 + lane;
     int kl = 0, kh = 31;
@@ -314,6 +326,7 @@ __global__ void __launch_bounds__(256) rows_kernel(uint32_t n, const float4 *__r
     const float4 ck = make_float4(__shfl_sync(0xffffffffu, cx, k), __shfl_sync(0xffffffffu, cy, k), 0.f, 0.f);
     const uint32_t slot = base + (uint32_t)qq;
     bool two = false;
+    uint32_t second = 0;
     if (qq < total && slot < cap) {
       int a0 = sx0, a1 = sx1, c0 = 1, c1 = 0;
       if (qk.ok) row_ranges(qk, ck, ty, W, H, sx0, sx1, tshift, a0, a1, c0, c1);
@@ -326,14 +339,29 @@ __global__ void __launch_bounds__(256) rows_kernel(uint32_t n, const float4 *__r
       if (a0 > a1) { a0 = 1; a1 = 0; }
       if (c0 > c1) { c0 = 1; c1 = 0; }
       two = c0 <= c1;
-      spans[slot] = make_uint2((uint32_t)a0 | ((uint32_t)a1 << 16), (uint32_t)c0 | ((uint32_t)c1 << 16));
+      spans[slot] = pack_range(a0, a1);
+      second = pack_range(c0, c1);
     }
-    split |= __reduce_or_sync(0xffffffffu, two ? 1u << k : 0u);
+    const uint32_t twos = __ballot_sync(0xffffffffu, two);
+    if (twos) {  // rare: each joins its surfel's chain
+      uint32_t at = 0;
+      if (lane == 0) {
+        at = atomicAdd(n_more, (uint32_t)__popc(twos));
+        if ((uint64_t)at + (uint64_t)__popc(twos) > more_cap) atomicOr(status, kStCapacity);
+      }
+      at = __shfl_sync(0xffffffffu, at, 0);
+      for (uint32_t t = twos; t; t &= t - 1u, ++at) {  // warp-uniform
+        const int src = __ffs((int)t) - 1, owner = __shfl_sync(0xffffffffu, k, src);
+        const uint32_t next = __shfl_sync(0xffffffffu, head, owner);
+        if (at >= more_cap) continue;
+        if (lane == src) more[at] = make_uint2(next, (uint32_t)ty << (2 * kColBits) | second);
+        if (lane == owner) head = at + 1u;
+      }
+    }
   }
   if (i < n && (bin || !bits))  // with a selection of its own the lists hold no unbinned surfel
     info[i] = make_uint4((uint32_t)rc.x | ((uint32_t)rc.y << 16), (uint32_t)rc.z | ((uint32_t)rc.w << 16),
-                         base + (uint32_t)(incl - nr),
-                         (bin ? kInfoBinned : 0u) | (((split >> lane) & 1u) ? kInfoSplit : 0u));
+                         base + (uint32_t)(incl - nr), (bin ? kInfoBinned : 0u) | head << 1);
   }
 }
 
@@ -393,7 +421,8 @@ struct ReuseApply {
 //
 //   row lists (one CTA per sub-chunk): per tile row, the tile ranges of the
 //     sub-chunk's surfels in that row, in depth order (a row with two ranges gives
-//     two entries, one that is empty an empty one), each with its surfel id;
+//     two entries, one that is empty an empty one), each with its surfel's place in
+//     the sub-chunk;
 //   mode 0 (CTA per (chunk, kCountRows rows)): each warp counts its lists' hits
 //     per tile; the 8 counts of a (tile, chunk) go to table[tile][chunk] as 8 x 16
 //     bits;
@@ -407,18 +436,22 @@ constexpr int kBandRows = 4;    // rows of a band (gs_usage counts (surfel, band
 static_assert(kBandRows == 4, "row_list_kernel finds a band's rows in a block's nibbles");
 constexpr int kCountRows = 4;   // rows a counting CTA takes
 
-// One (surfel, row range): surfel id, first column | last column << 16.
-struct RowEntry {
-  uint32_t id, range;
-};
+// One (surfel, row range) in 32 bits: the surfel's place in its sub-chunk above its
+// columns. The sub-chunk's ids (a few KB) stay in L1; with the id itself an entry takes
+// 8 bytes, and the pool has to hold as many entries as the eye has spans.
+using RowEntry = uint32_t;
 static_assert(sizeof(RowEntry) == kRowEntryBytes, "row entry layout");
+constexpr uint32_t kMaxWarpSurfels = 1u << (32 - 2 * kColBits);
+__device__ __forceinline__ RowEntry row_entry(uint32_t place, uint32_t range) { return place << (2 * kColBits) | range; }
+__device__ __forceinline__ uint32_t entry_place(RowEntry e) { return e >> (2 * kColBits); }
 
 struct ListArgs {
   const uint32_t *ids;     // depth-ordered binned surfels
   const uint32_t *n_vis;
   uint32_t n_max;
   const uint4 *info;       // per surfel: rectangle, slot of its first row in spans, flags (rows_kernel)
-  const uint2 *spans;      // tile ranges of every rectangle row (rows_kernel)
+  const uint32_t *spans;   // tile range of every rectangle row (rows_kernel)
+  const uint2 *more;       // the second ranges: next of the surfel plus one, row << 18 | range
   uint32_t span_cap;
   const uint16_t *clip;    // ROI mask: per row and column the next masked column, or null
   int tiles_x, tiles_y;
@@ -545,21 +578,18 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
     for (uint32_t g = g0; g < g1; ++g) {  // warp-uniform
       const uint32_t j = s0 + g * 32u + (uint32_t)lane;
       int y0 = 1, y1 = 0;
-      uint32_t id = 0, ro = 0;
+      uint32_t ro = 0;
       int x0 = 0, x1 = 0;
-      bool split = false;
+      uint32_t head = 0;
       uint4 inf = make_uint4(0u, 0u, 0u, 0u);
-      if (j < s1) {
-        id = a.ids[j];
-        inf = __ldg(a.info + id);
-      }
+      if (j < s1) inf = __ldg(a.info + a.ids[j]);
       if (inf.w & kInfoBinned) {
         x0 = (int)(inf.x & 0xffffu); y0 = (int)(inf.x >> 16);
         x1 = (int)(inf.y & 0xffffu); y1 = (int)(inf.y >> 16);
         ro = inf.z;
-        split = (inf.w & kInfoSplit) != 0u;
+        head = inf.w >> 1;
       }
-      const bool any_split = __any_sync(0xffffffffu, split);
+      const bool any_split = __any_sync(0xffffffffu, head != 0u);
       const bool has = y0 <= y1;
       const int ymin = __reduce_min_sync(0xffffffffu, has ? y0 : 0x7fffffff);
       const int ymax = __reduce_max_sync(0xffffffffu, has ? y1 : -1);
@@ -579,15 +609,12 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
         const uint32_t ca = transpose_bits(ra, lane);  // lane k: the surfels with an entry in row base + k
         uint32_t cb = 0;
         if (any_split) {  // and those with a second one (rare)
-          uint32_t t = split ? ra : 0u, rb = 0;
-          while (t) {
-            const int k = __ffs((int)t) - 1;
-            t &= t - 1u;
-            const uint32_t slot = ro + (uint32_t)(base + k - y0);
-            if (slot < a.span_cap) {
-              const uint2 sp = a.spans[slot];
-              rb |= (uint32_t)((sp.y & 0xffffu) <= (sp.y >> 16)) << k;
-            }
+          uint32_t rb = 0;
+          for (uint32_t h = head; h;) {
+            const uint2 m = __ldg(a.more + (h - 1u));
+            const uint32_t k = (m.y >> (2 * kColBits)) - (uint32_t)base;
+            if (k < 32u) rb |= 1u << k;
+            h = m.x;
           }
           any_rb |= __any_sync(0xffffffffu, rb != 0u) ? 1u : 0u;
           cb = transpose_bits(rb, lane);
@@ -609,11 +636,15 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
         for (int y = y0; y <= y1; ++y) {
           const uint32_t m = col[y];
           const uint32_t slot = ro + (uint32_t)(y - y0);
-          const uint2 sp = (m & bit) && slot < a.span_cap ? __ldg(a.spans + slot) : make_uint2(1u, 1u);
+          const uint32_t sp = (m & bit) && slot < a.span_cap ? __ldg(a.spans + slot) : kNoRange;
           uint32_t at = cnt[y] + (uint32_t)__popc(m & lt);
           if (any_rb) at += (uint32_t)__popc(colb[y] & lt);
-          if ((m & bit) && at < a.pool_cap) a.pool[at] = RowEntry{id, sp.x};
-          if (any_rb && (colb[y] & bit) && at + 1u < a.pool_cap) a.pool[at + 1u] = RowEntry{id, sp.y};
+          if ((m & bit) && at < a.pool_cap) a.pool[at] = row_entry(j - s0, sp);
+          if (any_rb && (colb[y] & bit) && at + 1u < a.pool_cap) {
+            uint2 m2 = __ldg(a.more + (head - 1u));
+            while ((int)(m2.y >> (2 * kColBits)) != y) m2 = __ldg(a.more + (m2.x - 1u));  // the row is in the chain
+            a.pool[at + 1u] = row_entry(j - s0, m2.y & ((1u << 2 * kColBits) - 1u));
+          }
         }
         __syncwarp();
         for (int blk = blk0; blk <= blk1; ++blk) {
@@ -633,11 +664,12 @@ __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
 struct BinArgs {
   const uint32_t *n_vis;   // binned surfels (device)
   uint32_t n_max;
+  const uint32_t *ids;     // depth-ordered binned surfels
   const RowEntry *pool;
   const uint2 *lists;      // [chunk][row][warp]
   const uint8_t *mask;     // ROI tile mask, or null
   int tiles_x, tiles_y;
-  uint32_t warp_surfels;   // surfels per warp sub-chunk (< 65536)
+  uint32_t warp_surfels;   // surfels per warp sub-chunk
   uint32_t nch;            // chunks (row length of the tables)
   uint4 *table;            // [tile][chunk] 8 x 16-bit per-warp counts
   const uint32_t *offs;    // [tile][chunk] exclusive offsets (mode 1)
@@ -679,13 +711,13 @@ __global__ void __launch_bounds__(kBinThreads) bin_count_kernel(BinArgs a) {
     const RowEntry *q = a.pool + li[r].x;
     for (uint32_t e = (uint32_t)lane; e < li[r].y; e += 32) {
       const RowEntry en = q[e];
-      const int c0 = (int)(en.range & 0xffffu), c1 = (int)(en.range >> 16);
+      const int c0 = range_lo(en), c1 = range_hi(en);
       atomicAdd(&d[c0], 1u);
       atomicSub(&d[c1 + 1], 1u);
       if (a.cnt_bin) {
         uint32_t n = 0;
         for (int x = c0; x <= c1; ++x) n += !a.mask || a.mask[(size_t)(y0 + r) * tx_n + x] != 0;
-        if (n) atomicAdd(&a.cnt_bin[en.id], n);
+        if (n) atomicAdd(&a.cnt_bin[a.ids[(c * kBinWarps + w) * a.warp_surfels + entry_place(en)]], n);
       }
     }
     __syncwarp();
@@ -724,10 +756,17 @@ __global__ void __launch_bounds__(kBinThreads) bin_count_kernel(BinArgs a) {
 // the launch. 1.5M / 3M surfels at 1920x1080 / 2448x2448: 44 / 105 us, against 94 /
 // 243 for an instance per lane ranked by shared-memory masks; collecting a CTA's
 // instances in shared memory for coalesced copies measured 53 / 112.
+// An entry's id is one more gather behind the entry: it goes to shared memory by
+// cp.async a step ahead, the first beside the counts' loads (loaded to a register with
+// the entry it cost 3 us of the 660 of the 500k-surfel frame).
+__device__ __forceinline__ void cp_async4(uint32_t *dst, const uint32_t *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
 __global__ void __launch_bounds__(kBinThreads, 8) bin_place_kernel(BinArgs a) {
   griddep_wait();
   extern __shared__ uint32_t s_cnt[];  // [kBinWarps][tiles_x]: every warp's next slot per tile
-  __shared__ uint32_t s_id[kBinWarps][32];
+  __shared__ uint32_t s_id[2][kBinWarps][32];
   __shared__ uint32_t s_mask[(kMaxTileCols + 31) / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const uint32_t nv = load_n(a.n_vis, a.n_max);
@@ -737,7 +776,12 @@ __global__ void __launch_bounds__(kBinThreads, 8) bin_place_kernel(BinArgs a) {
   const int ty = (int)blockIdx.y;
   const size_t t0 = (size_t)ty * tx_n;  // first tile of the row
   const uint2 li = a.lists[((size_t)c * a.tiles_y + ty) * kBinWarps + w];
-  if (!__syncthreads_or(li.y > 0u)) return;  // nothing reaches the row
+  const RowEntry *q = a.pool + li.x;
+  const int qn = (int)li.y;
+  const uint32_t *ids = a.ids + (size_t)(c * kBinWarps + w) * a.warp_surfels;
+  RowEntry next = lane < qn ? q[lane] : kNoRange;
+  if (!__syncthreads_or(qn > 0)) return;  // nothing reaches the row
+  if (lane < qn) cp_async4(&s_id[0][w][lane], ids + entry_place(next));
   for (int bt = tid; bt < tx_n; bt += kBinThreads) {
     const size_t e = (t0 + bt) * a.nch + c;
     const uint4 v = a.table[e];
@@ -757,18 +801,13 @@ __global__ void __launch_bounds__(kBinThreads, 8) bin_place_kernel(BinArgs a) {
   }
   __syncthreads();
   uint32_t *my_cnt = s_cnt + w * tx_n;
-  const RowEntry *q = a.pool + li.x;
-  const int qn = (int)li.y;
-  RowEntry next{0u, 1u};  // columns [1, 0]: none
-  if (lane < qn) next = q[lane];
-  for (int qpos = 0; qpos < qn; qpos += 32) {  // warp-uniform
+  for (int qpos = 0, buf = 0; qpos < qn; qpos += 32, buf ^= 1) {  // warp-uniform
     const RowEntry en = next;
     const int e = qpos + 32 + lane;  // the next step's entries are fetched a step ahead
-    next = e < qn ? q[e] : RowEntry{0u, 1u};
-    __syncwarp();  // the previous step's ids have been read
-    s_id[w][lane] = en.id;
-    __syncwarp();
-    const int c0 = (int)(en.range & 0xffffu), c1 = (int)(en.range >> 16);
+    next = e < qn ? q[e] : kNoRange;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();  // the step's ids are there, and those of the step before have been read
+    const int c0 = range_lo(en), c1 = range_hi(en);
     const int lo = __reduce_min_sync(0xffffffffu, c0 <= c1 ? c0 : 0x7fffffff);
     const int hi = __reduce_max_sync(0xffffffffu, c0 <= c1 ? c1 : -1);
     for (int base = lo & ~31; base <= hi; base += 32) {  // warp-uniform
@@ -778,7 +817,7 @@ __global__ void __launch_bounds__(kBinThreads, 8) bin_place_kernel(BinArgs a) {
       if (m) {  // the lane's column is in the row: no other lane touches its counter
         uint32_t pos = my_cnt[base + lane];
         do {
-          const uint32_t id = s_id[w][__ffs((int)m) - 1];
+          const uint32_t id = s_id[buf][w][__ffs((int)m) - 1];
           m &= m - 1u;
           if (pos < a.cap) {
             a.ival[pos] = id;
@@ -789,6 +828,7 @@ __global__ void __launch_bounds__(kBinThreads, 8) bin_place_kernel(BinArgs a) {
         my_cnt[base + lane] = pos;
       }
     }
+    if (e < qn) cp_async4(&s_id[buf ^ 1][w][lane], ids + entry_place(next));
   }
 }
 
@@ -850,7 +890,7 @@ uint32_t bin_warp_surfels(int max_surfels) {
   const uint32_t per = ((uint32_t)max_surfels + kBinWarps * 256 - 1) / (kBinWarps * 256);
   uint32_t r = (per + 31) / 32 * 32;
   if (r < 64) r = 64;
-  if (r > 32768) r = 32768;  // per-warp counts are 16-bit
+  if (r > kMaxWarpSurfels) r = kMaxWarpSurfels;  // (and the per-warp counts are 16-bit)
   return r;
 }
 
@@ -904,7 +944,7 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   if (tile_mask) {  // (the rasterizer-grid mask and) its summed-area table
     launch_k(mask_sat_kernel, 1, 1024, 0, s, const_cast<uint8_t *>(tile_mask), tiles_x, tiles_y, b.mask_sat, roi16,
              (W + kTile - 1) / kTile, (H + kTile - 1) / kTile, roi16 ? tshift : 4, b.mask_clip,
-             roi16 ? b.items16 : nullptr, &ctr->n_rows[eye]);
+             roi16 ? b.items16 : nullptr, &ctr->n_rows[eye], &ctr->n_more[eye]);
     GS_LAUNCHED(1);
   }
   // 1. the row spans. A full binning's need only the preprocessed records: on a
@@ -922,8 +962,8 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
     const int grid = cap_g < (n + 255) / 256 ? cap_g : (n + 255) / 256;
     GS_LAUNCHED(1);
     return launch_k(rows_kernel, grid, 256, 0, st, (uint32_t)n, ws.rec[eye], ws.rect[eye], ws.vis[eye], ws.cams, eye,
-                    ws.prim, ws.info[eye], ws.spans[eye], cap, &ctr->n_rows[eye], &ctr->status,
-                    tile_mask ? b.mask_clip : nullptr, tiles_x, tiles_y, tile_mask ? b.mask_sat : nullptr,
+                    ws.prim, ws.info[eye], ws.spans[eye], cap, &ctr->n_rows[eye], ws.more[eye], ws.more_cap[eye],
+                    &ctr->n_more[eye], &ctr->status, tile_mask ? b.mask_clip : nullptr, tiles_x, tiles_y, tile_mask ? b.mask_sat : nullptr,
                     tile_mask ? b.bits : nullptr);
   };
   if (!side && (err = launch_rows(s)) != cudaSuccess) return err;
@@ -955,6 +995,7 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   la.n_max = (uint32_t)n;
   la.info = ws.info[eye];
   la.spans = ws.spans[eye];
+  la.more = ws.more[eye];
   la.span_cap = cap;
   la.clip = tile_mask ? b.mask_clip : nullptr;
   la.tiles_x = tiles_x;
@@ -971,6 +1012,7 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   BinArgs a;
   a.n_vis = &ctr->n_vis[eye];
   a.n_max = (uint32_t)n;
+  a.ids = b.dval[0];
   a.pool = b.row_pool;
   a.lists = b.row_lists;
   a.mask = tile_mask;

@@ -69,6 +69,7 @@ struct Counters {
   uint32_t n_rects;      // centre components found
   uint32_t n_sort[2];    // instances actually binned per eye (capacity-clamped)
   uint32_t n_rows[2];    // (surfel, tile row) spans per eye
+  uint32_t n_more[2];    // of which have a second range
   uint32_t n_band[2];    // (surfel, band of 4 tile rows) pairs of the last binning per eye
   uint32_t n_entries[2]; // row list entries of the last binning per eye
   uint32_t n_items[2];   // rasterizer tiles listed by the last masked binning per eye
@@ -98,7 +99,7 @@ struct BinScratch {
   uint32_t *dkey[2], *dval[2];  // depth sort double buffers; the depth order ends in dval[0]
   uint32_t *bits;               // an ROI binning's surfels, one bit each
   uint4 *bin_table;             // [tile][chunk] per-warp instance counts (8 x 16 bits)
-  struct RowEntry *row_pool;    // (surfel, row range) entries of every warp's lists
+  uint32_t *row_pool;           // (surfel, row range) entries of every warp's lists
   uint2 *row_lists;             // [chunk][row][warp]: first entry, entries
   uint32_t *bin_offs;           // their tile-major exclusive scan
   uint32_t *ival;               // surfel id per instance, grouped by tile, depth order inside
@@ -129,13 +130,14 @@ struct Workspace {
   uint32_t *zkey[2];            // float bits of the centre depth per surfel and eye
   uint32_t *vis[2];             // one bit per surfel and eye: its rectangle is not empty
   uint32_t *cnt_bin;            // tiles each surfel reaches in the last binning (keep_intermediates)
-  uint32_t row_pool_cap[2];     // entries of row_pool, per eye
+  uint32_t row_pool_cap[2], more_cap[2];  // entries of row_pool and of more, per eye
   BinScratch bin[2];            // per eye
   uint8_t *tile_mask;           // ROI mask on the 16-pixel grid
   uint8_t *strip_mask;          // edge-strip tiles of a reused depth range (16-pixel grid)
   float *strip_rgb;             // [3][pixels] the affiliated eye's strip tiles, rendered ahead
   uint4 *info[2];               // per surfel and eye: rectangle, slot of its first row in spans, flags
-  uint2 *spans[2];              // per (surfel, tile row): tile ranges [a0, a1] u [c0, c1], 4 x 16 bits
+  uint32_t *spans[2];           // per (surfel, tile row): its (first) range of tile columns
+  uint2 *more[2];               // second ranges, a surfel's chained from its info
   // scans outside the binning (centre ROIs, repair tile lists) use bin[0]'s scratch
   unsigned long long *warpbuf;
   float *warp_depth;
@@ -226,7 +228,7 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
 uint32_t bin_warp_surfels(int max_surfels);
 uint32_t bin_chunks(int max_surfels);
 size_t row_list_words(int max_surfels, int max_tiles_y);
-constexpr size_t kRowEntryBytes = 8;
+constexpr size_t kRowEntryBytes = 4;
 cudaError_t prepare_binning(int max_tiles_x, int max_tiles_y);
 // ---- learned repair network ----
 constexpr int kRepairParams = 39908;

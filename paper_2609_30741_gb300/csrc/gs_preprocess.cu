@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kSetupThreads) setup_cams_kernel(PoseArgs pa, 
     ctr->n_inst[e] = 0;
     ctr->n_sort[e] = 0;
     ctr->n_rows[e] = 0;
+    ctr->n_more[e] = 0;
     ctr->n_band[e] = 0;
     ctr->n_entries[e] = 0;
     ctr->n_items[e] = 0;
