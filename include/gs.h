@@ -441,12 +441,13 @@ gs_status gs_centre_rois(gs_context *ctx, const uint8_t *cls, int width, int hei
  *   tile  8, 16 or 32: edge of the rasterizer's square tiles, pixels; at least
  *         the context's min_tile. The ROI generator keeps the 16-pixel grid:
  *         with 32-pixel tiles only the pixels of ROI 16-pixel tiles are written.
- *   pix   pixels per thread, i.e. the block shape (tile^2 / pix threads): 1 or 2
- *         at tile 8, 2 or 4 at tile 16, 2, 4 or 8 at tile 32.
- *   batch 32, 64, 128 or 256 surfel records per shared-memory stage.
+ *   pix   pixels per thread: 1 or 2 at tile 8, 2 or 4 at tile 16, 2, 4 or 8 at
+ *         tile 32. At tiles 16 and 32 the values run the same kernel, which blends
+ *         16-pixel squares and chooses its block shape by their number.
+ *   batch 32, 64, 128 or 256 surfel records per shared-memory stage; 64, 128 and
+ *         256 run the same kernel, with stages of 64.
  * Every configuration produces the same images bit for bit; they differ in
- * speed only. (The rasterizer may use another block shape or a shorter stage
- * where it is faster; 16- and 32-pixel tiles are blended in 16-pixel squares.) The default is {16, 4, 128} ({32, 8, 128} when min_tile = 32).
+ * speed only. The default is {16, 4, 128} ({32, 8, 128} when min_tile = 32).
  * Returns GS_ERR_BAD_ARG for any other value. */
 typedef struct {
   int tile, pix, batch;
@@ -542,8 +543,9 @@ gs_status gs_render_mono_batch(gs_batch *b, const gs_mono_frame *frames, int n_f
  * the slots allow (two untimed calls, then `reps` calls timed with CUDA events
  * on the call's stream; the median counts) and leaves the fastest set on the
  * batch / context. results[0..*n_results) gets
- * every configuration tried with its median ms (-1: the configuration
- * overflowed a buffer or failed). Results are cached for the process under a
+ * every configuration the slots allow with its median ms (-1: the configuration
+ * overflowed a buffer or failed); those that run the same kernel are timed once
+ * and share it. Results are cached for the process under a
  * key of the GPU (name, compute capability, SM count) and the frames' shapes
  * (image size, surfel-count power-of-two bucket, SH degree; stereo with plain
  * or learned repair, or two-pass); with use_cache = 1 a cached entry is applied without timing

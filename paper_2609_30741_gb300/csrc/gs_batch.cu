@@ -597,7 +597,8 @@ gs_status gs_render_two_pass_batch(gs_batch *b, const gs_frame *frames, int n_fr
 // `apply` accepts: two untimed calls (the first enqueues kernel by kernel, the
 // second captures the graph), then `reps` calls, each between CUDA events; the
 // median is the configuration's time. A configuration whose calls fail or
-// overflow a device buffer gets ms = -1.
+// overflow a device buffer gets ms = -1. One that runs the kernel of an earlier one
+// gets that one's time: timed apart, noise would choose among them.
 template <class Apply, class Call, class Check>
 static gs_status tune_loop(cudaStream_t s, int reps, int min_tshift, Apply &&apply, Call &&call, Check &&check,
                            gs_tune_result *results, int max_results, int *n_results, gs_raster_config *best,
@@ -607,6 +608,7 @@ static gs_status tune_loop(cudaStream_t s, int reps, int min_tshift, Apply &&app
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return BFAIL(cudaGetLastError());
   std::vector<float> t(reps);
+  std::vector<gs_tune_result> done;
   int nr = 0;
   gs_raster_config win{0, 0, 0};
   float win_ms = INFINITY;
@@ -615,8 +617,20 @@ static gs_status tune_loop(cudaStream_t s, int reps, int min_tshift, Apply &&app
     for (int bi = 0; bi < 4 && err == GS_OK; ++bi) {
       const gs_raster_config rc{shapes[si][0], shapes[si][1], batches[bi]};
       if (raster_tshift(RasterConfig{rc.tile, rc.pix, rc.batch}) < min_tshift) continue;
-      if (apply(rc) != GS_OK) continue;
       float ms = -1.f;
+      bool known = false;
+      for (const gs_tune_result &d : done)
+        if (raster_same(RasterConfig{d.rc.tile, d.rc.pix, d.rc.batch}, RasterConfig{rc.tile, rc.pix, rc.batch})) {
+          known = true;
+          ms = d.ms;
+          break;
+        }
+      if (known) {
+        if (results && nr < max_results) results[nr] = gs_tune_result{rc, ms};
+        ++nr;
+        continue;
+      }
+      if (apply(rc) != GS_OK) continue;
       gs_status st = call();
       if (st == GS_OK) st = call();
       int dev = GS_OK;
@@ -639,6 +653,7 @@ static gs_status tune_loop(cudaStream_t s, int reps, int min_tshift, Apply &&app
           win = rc;
         }
       }
+      done.push_back(gs_tune_result{rc, ms});
       if (results && nr < max_results) results[nr] = gs_tune_result{rc, ms};
       ++nr;
     }

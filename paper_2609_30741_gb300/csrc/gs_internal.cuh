@@ -306,8 +306,9 @@ struct RasterTable {
   RasterFrame f[kRasterFrames];
   int n;
 };
-// Tile edge, pixels per thread (the block has tile^2 / pix threads) and surfel
-// records per shared-memory stage.
+// Tile edge, pixels per thread and surfel records per shared-memory stage, as the
+// caller gave them. The kernel follows from the tile edge, at 8 pixels also from pix,
+// and from whether the stage is 32 records or more (raster_same: 8 kernels in all).
 struct RasterConfig {
   int tile, pix, batch;
 };
@@ -321,6 +322,7 @@ inline int sm_grid_cap(int per_sm) {
 }
 bool raster_config_ok(const RasterConfig &c);
 int raster_tshift(const RasterConfig &c);
+bool raster_same(const RasterConfig &a, const RasterConfig &b);  // the same tile grid and kernel
 // `queue` holds two words that are zero between launches (the launch's last CTA
 // clears them).
 cudaError_t launch_raster(const RasterTable &t, const RasterConfig &c, bool count_pairs, uint32_t *queue,

@@ -642,6 +642,10 @@ bool raster_config_ok(const RasterConfig &c) { return shape_index(c) >= 0 && bat
 
 int raster_tshift(const RasterConfig &c) { return c.tile == 8 ? 3 : c.tile == 32 ? 5 : 4; }
 
+bool raster_same(const RasterConfig &a, const RasterConfig &b) {
+  return a.tile == b.tile && shape_index(a) == shape_index(b) && batch_index(a.batch) == batch_index(b.batch);
+}
+
 cudaError_t launch_raster(const RasterTable &t, const RasterConfig &c, bool count_pairs, uint32_t *queue,
                           cudaStream_t s) {
   if (!raster_config_ok(c) || t.n < 0 || t.n > kRasterFrames) return cudaErrorInvalidValue;
