@@ -19,8 +19,9 @@ int g_pdl = 1;
 namespace {
 
 constexpr size_t kAlign = 256;
-// widest image: the binning keeps 8 warps x 4 tile rows x 1 counter per tile
-// column in shared memory (64 KB at kMaxTileCols), and per tile row 8 counters
+// widest and tallest image: the binning keeps 8 warps x 4 tile rows x 1 counter per
+// tile column in shared memory (64 KB at kMaxTileCols), and 8 warps x (1 counter and 2
+// column masks) per tile row (96 KB at the 1024 rows of 8-pixel tiles)
 constexpr int kMaxWidth = 8192;
 
 struct Carver {
@@ -502,7 +503,6 @@ static void mark(gs_context *ctx, int slot) {
   ctx->nmarks = slot + 1 > ctx->nmarks ? slot + 1 : ctx->nmarks;
 }
 
-// One eye through the persistent rasterizer (a table of one frame).
 // The stream and events on which a binning computes its row spans beside its
 // depth order (created on first use); null if they cannot be.
 static const SideRows *side_rows(gs_context *ctx) {
@@ -904,12 +904,8 @@ static gs_status stereo_impl(gs_context *ctx, const gs_scene *scene, const gs_po
     // on their own grid)
     ctx->last_tiles = tx * ty;
     const int aorder = p.parallel ? kOrderReuse : kOrderOwn;
-    // (with depth_mode 2 the strip binning of this eye ran on the second stream:
-    // its spans stay in stream order)
-    const SideRows *sr = reuse ? nullptr : side_rows(ctx);
-    e = sh != 4 ? launch_binning(ws, 1, scene->n, tx, ty, ws.bin[1].rmask, ctx->stream, aorder, ws.tile_mask, W, H, sh,
-                                 sr)
-                : launch_binning(ws, 1, scene->n, tx, ty, ws.tile_mask, ctx->stream, aorder, nullptr, 0, 0, 4, sr);
+    e = sh != 4 ? launch_binning(ws, 1, scene->n, tx, ty, ws.bin[1].rmask, ctx->stream, aorder, ws.tile_mask, W, H, sh)
+                : launch_binning(ws, 1, scene->n, tx, ty, ws.tile_mask, ctx->stream, aorder);
     if (e != cudaSuccess) return cuda_fail(e);
     mark(ctx, 6);
     RasterFrame rf = roi_frame(ws.tile_mask, out->rgb_aff, ws.cls);

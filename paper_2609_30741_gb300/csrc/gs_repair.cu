@@ -17,20 +17,20 @@
 // cores. Activations stay in shared memory in the canonical no-swizzle K-major
 // layout [channel group][position][8 channels]; a 3x3 tap is just a shift of the
 // A operand's start address along the 28-wide grid, so no im2col copy exists.
-// One thread issues tcgen05.mma (M = 128 positions, N = 32 channels, K = 16)
-// into tensor memory; four warps read the accumulators back, add the bias,
-// apply ReLU and the image-border zeroing, and store BF16 for the next layer.
+// One warp issues tcgen05.mma (M = 128 positions, N = 32 channels, K = 16) into
+// tensor memory; eight warps read the accumulators back, add the bias, apply ReLU
+// and the image-border zeroing, and store BF16 for the next layer.
 //
 // Training runs the same forward kernel (keeping every layer's input), then a
 // loss kernel, and per layer (last to first) one backward kernel on the tensor
 // cores: the input gradient is the full convolution of the output gradient with
 // the flipped, transposed weights (the forward's implicit GEMM with another
 // weight image and the ReLU derivative in the epilogue), and the weight
-// gradient is a GEMM over positions per 3x3 tap (M = c_out, N = c_in, K = the
-// tile's positions, the tap again a shift of an operand's start address),
-// accumulated in tensor memory over all tiles a CTA takes; the CTAs' partial
-// sums are reduced in a fixed order (no atomics, so a step is deterministic).
-// AdamW updates the FP32 master weights.
+// gradient is a GEMM over positions per row of 3x3 taps (M = three taps x c_out,
+// N = c_in, K = the tile's positions, the taps again shifts of an operand's start
+// address), accumulated in tensor memory over all tiles a CTA takes. One kernel
+// adds the CTAs' partial sums in a fixed order (no atomics, so a step is
+// deterministic) and applies AdamW to the FP32 master weights.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 
@@ -881,7 +881,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   constexpr int NW = l == 0 ? 16 : 32;            // weight-gradient N: c_in padded to 16
   constexpr int nK = kchunks(l);
   constexpr int MT = l > 0 ? mtiles(l - 1) : 0;   // input-gradient M tiles: layer l's input window
-  constexpr int vin = kGW - 2 * l, vout = vrows(l);
+  constexpr int vin = kGW - 2 * l;
   constexpr int kg = kgd(l);
   constexpr int gD = (co_n + 7) / 8;                   // c_out groups that are not zero
   constexpr int gX = l == 0 ? 1 : 4;                   // c_in groups stored
