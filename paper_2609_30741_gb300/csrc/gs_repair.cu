@@ -830,7 +830,8 @@ struct BwdArgs {
                            // 16 kchunks(l) positions, zero outside the window
   uint4 *dyo;              // [n][4][kNPos]: BF16 dL/d(output of layer l - 1) (l >= 1)
   const uint8_t *wpackT;   // the transposed image of layer l
-  float *part;             // [gridDim][cout(l) * 9 * cin(l) + cout(l)] weight and bias gradients per CTA
+  float *part;             // weight and bias gradients of CTA b at part + b * part_stride: see kPartAct
+  size_t part_stride;
   int n;
   uint32_t *status;
 };
@@ -1083,7 +1084,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
     // stored [tap][c_in][c_out], so a warp's stores are whole lines (in the parameters' own
     // order they were 32 lines each and took 17k cycles)
     constexpr int npar = co_n * 9 * ci_n;
-    float *part = a.part + (size_t)blockIdx.x * (npar + co_n);
+    float *part = a.part + (size_t)blockIdx.x * a.part_stride;
     const int co = lane;
 #pragma unroll 1
     for (int u = wg; u < 3 * (NW / 16); u += 2) {
@@ -1104,8 +1105,15 @@ __global__ void __launch_bounds__(kBwdThreads, 1) repair_bwd_kernel(BwdArgs a) {
   if (wid == 0) umma::tmem_dealloc(taddr, kBwdTmemCols);
 }
 
+// The partial gradients of layer l < 5 lie where the forward kept layer l + 1's input,
+// which the backward has done with: CTA b's in tile b's (a CTA takes a tile at least).
+// A buffer of their own for all layers took 24 MB.
+constexpr size_t kActFloats = (size_t)6 * 4 * kNPos * 4;  // of a tile, and of layer l's input in it:
+__host__ __device__ constexpr size_t kPartAct(int l) { return (size_t)(l + 1) * 4 * kNPos * 4; }
+static_assert(poff(2) - poff(1) <= 4 * kNPos * 4 && poff(1) - poff(0) <= 4 * kNPos * 4, "a layer's partials fit its input");
+
 struct UpdateArgs {
-  const float *part;  // per layer [n_parts][its parameters], layers in order
+  const float *part5, *acts;  // the CTAs' partials of layer 5, and where those of layers 0-4 lie (kPartAct)
   int n_parts;
   float *grad, *w, *m, *v;
   float lr, b1, b2, eps, wd, bc1, bc2;  // AdamW, with lr > 0
@@ -1123,22 +1131,22 @@ __global__ void __launch_bounds__(256) repair_update_kernel(UpdateArgs a) {
   int par = i;                           // the parameter
   float sum = 0.f;
   if (i < kRepairParams) {
-    int off = poff(0), end = poff(1), ci_n = cin(0), co_n = cout(0);
+    int l = 0, off = poff(0), ci_n = cin(0), co_n = cout(0);
 #pragma unroll
     for (int k = 1; k < 6; ++k)
       if (i >= poff(k)) {
+        l = k;
         off = poff(k);
-        end = poff(k + 1);
         ci_n = cin(k);
         co_n = cout(k);
       }
     // the partials lie [tap][c_in][c_out], the parameters [c_out][tap][c_in]; biases last in both
     const int e = i - off, co = e % co_n, rest = e / co_n;
     if (e < co_n * 9 * ci_n) par = off + (co * 9 + rest / ci_n) * ci_n + rest % ci_n;
-    const int count = end - off;
-    const float *p = a.part + (size_t)a.n_parts * off + (i - off);
+    const size_t stride = l == 5 ? (size_t)(poff(6) - poff(5)) : kActFloats;
+    const float *p = (l == 5 ? a.part5 : a.acts + kPartAct(l)) + (i - off);
 #pragma unroll 8
-    for (int k = wid; k < a.n_parts; k += 8) sum += __ldg(p + (size_t)k * count);
+    for (int k = wid; k < a.n_parts; k += 8) sum += __ldg(p + (size_t)k * stride);
   }
   s_sum[wid][lane] = sum;
   __syncthreads();
@@ -1165,9 +1173,9 @@ static int bwd_grid(int n) {
 size_t repair_train_scratch_bytes(int n_tiles) {
   const size_t n = (size_t)(n_tiles > 0 ? n_tiles : 1);
   // activations, raw outputs, gate, two BF16 gradient buffers, tile stats, the
-  // loss sums and the CTAs' partial gradients
+  // loss sums and the CTAs' partial gradients of the last layer
   return n * (repair_act_bytes_per_tile() + 4 * kRT * kRT * 4 + 4 + 2 * 4 * kNPos * 16 + 32) +
-         (size_t)bwd_grid((int)n) * kRepairParams * 4 + 10 * 256;  // + alignment of the 8 buffers
+         (size_t)bwd_grid((int)n) * (poff(6) - poff(5)) * 4 + 10 * 256;  // + alignment of the 8 buffers
 }
 
 using BwdKernel = void (*)(BwdArgs);
@@ -1297,7 +1305,7 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
   float *stats = (float *)take((size_t)n * 32);
   float *sums = (float *)take(8 * sizeof(float));
   const int G = bwd_grid(n);
-  float *part = (float *)take((size_t)G * kRepairParams * 4);
+  float *part5 = (float *)take((size_t)G * (poff(6) - poff(5)) * 4);
   if ((e = cudaMemsetAsync(sums, 0, 8 * sizeof(float), s)) != cudaSuccess) return e;
   if ((e = repair_forward(ws, b.feat, b.W, b.H, b.tiles, nullptr, (uint32_t)n, nullptr, gate, out4, acts, s, false,
                           nullptr)) != cudaSuccess)
@@ -1331,7 +1339,8 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
     ba.dy = cur;
     ba.dyo = nxt;
     ba.wpackT = ws.rp_wpackT;
-    ba.part = part + (size_t)G * poff(l);
+    ba.part = l == 5 ? part5 : (float *)acts + kPartAct(l);
+    ba.part_stride = l == 5 ? (size_t)(poff(6) - poff(5)) : kActFloats;
     ba.n = n;
     ba.status = &ws.ctr->status;
     launch_k(bwd_kernel(l), G, kBwdThreads, bwd_smem(), s, ba);
@@ -1341,7 +1350,8 @@ cudaError_t repair_train_step(const Workspace &ws, const RepairBatch &b, const R
     nxt = tmp;
   }
   UpdateArgs u;
-  u.part = part;
+  u.part5 = part5;
+  u.acts = (const float *)acts;
   u.n_parts = G;
   u.grad = ws.rp_grad;
   u.w = ws.rp_master;
