@@ -956,9 +956,11 @@ cudaError_t launch_binning(const Workspace &ws, int eye, int n, int tiles_x, int
   const auto launch_rows = [&](cudaStream_t st) -> cudaError_t {
     if (n <= 0) return cudaSuccess;
     // beside the sort a small grid leaves its latency-bound passes their SMs; with
-    // more surfels the spans are the longer branch, and a third CTA per SM pays
-    // (list start, 2 / 3 per SM: 500k surfels 121 / 125 us, 1.5M 249 / 240, 3M 479 / 444)
-    const int cap_g = sm_grid_cap(side && sort ? (n > (1 << 20) ? 3 : 2) : 6);
+    // more surfels the spans are the longer branch, and a third CTA per SM pays. Mono
+    // frames with 2 / 3 per SM, us: object scene 425 / 429 at 500k surfels, 495 / 495 at
+    // 750k, 567 / 553 at 1M, 646 / 621 at 1.25M; unbounded scene 418 / 424 at 750k,
+    // 488 / 483 at 1M, 615 / 605 at 1.5M, 806 / 779 at 2.2M
+    const int cap_g = sm_grid_cap(side && sort ? (n > 875000 ? 3 : 2) : 6);
     const int grid = cap_g < (n + 255) / 256 ? cap_g : (n + 255) / 256;
     GS_LAUNCHED(1);
     return launch_k(rows_kernel, grid, 256, 0, st, (uint32_t)n, ws.rec[eye], ws.rect[eye], ws.vis[eye], ws.cams, eye,
