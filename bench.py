@@ -9,7 +9,8 @@ the host cores instead (a bounded sample per step, extrapolated to a frame).
 
 Launch: python bench.py [--gpus N --steps K --warmup W]; for N > 1 under
 torch.distributed.run every rank renders its own frames (replicas, no
-collective on the data path) and rank 0 prints the JSON line.
+collective on the data path) and rank 0 prints the JSON line, in brief (numbers to
+six digits, no lists per frame); --detail FILE keeps the whole record.
 """
 from __future__ import annotations
 
@@ -44,27 +45,27 @@ PSNR_GATE_MIP = PSNR_FLOOR_MIP - 10 * math.log10(10 ** 0.13 - 1)
 #   (pixel, surfel) pair, counted against the FP32 lane rate;
 # - preprocess: 232 B of SH3 attributes read, two 64 B blend records and 8 B of
 #   tile counts written per surfel;
-# - binning: 12 B emitted, 6 sort passes of 24 B and 8 B of histogram per
-#   (surfel, tile) instance (the duplicate-and-sort binning of the tile
-#   rasterizer; the counting sort here moves fewer bytes than that);
-# - warp + classification: 84 B per pixel (read 20, clear 8, atomic 8, resolve
-#   8 + 20 gather + 20 write);
+# - binning: what it cannot do without. Per surfel 48 B of its record, its
+#   rectangle and its depth key read (60 B), per (surfel, tile) instance its id
+#   written (4 B). A floor: the kernels are a chain bound by latency;
+# - warp + classification: per pixel the warp reads depth and transmittance (8)
+#   and writes a key (8); the classification reads the key (8), gathers RGB (12)
+#   and writes RGB, depth and class (17);
 # - repair network: 79,488 FLOP per pixel over each candidate tile and its
 #   6-pixel halo (28 x 28 positions).
 OPS_PER_PAIR = 42
 PREPROCESS_BYTES_PER_SURFEL = 232 + 2 * 64 + 8
-BIN_BYTES_PER_INSTANCE = 12 + 6 * 24 + 8
-WARP_BYTES_PER_PIXEL = 84
+BIN_BYTES_PER_SURFEL, BIN_BYTES_PER_INSTANCE = 60, 4
+WARP_BYTES_PER_PIXEL = 8 + 8 + 8 + 12 + 17
 REPAIR_FLOP_PER_PIXEL = 79488
 REPAIR_WINDOW_PX = 28 * 28
-# The rasterizer's own instruction count (for comparison): per evaluated pair
-# the row offset and the three plane-point FMAs (4), reciprocal, u and v (3),
-# rho3 (2), rho2 (2), min and the threshold compare (2) = 13, the live-bit test
-# (3) and a 1/pix share of the per-surfel column set-up (dx, its three plane
-# terms and dx^2: 5) that a thread's pix pixels share; and per contributing
-# pair: exponent fma, ex2, alpha clamp, T update, stop compare, depth (2 fma +
-# select), weight, RGB and depth accumulation (4) = 12.
-OPS_EVAL_PIXEL, OPS_EVAL_COLUMN, OPS_CONTRIB = 16, 5, 12
+# The rasterizer's own operations (for comparison), two records packed in one
+# FP32x2 instruction counted as two. Per evaluated pair: row offset and three
+# plane-point FMAs (4), reciprocal, u and v (3), rho (2), depth (2), exponent (2),
+# ex2, alpha clamp, support compare, T, weight, stop compare (6) = 19; a share of
+# the column's dx and plane terms (4, over the thread's two pixels at 16- and
+# 32-pixel tiles); per contributing pair RGB, depth and T (5).
+OPS_EVAL_PIXEL, OPS_EVAL_COLUMN, OPS_CONTRIB = 19, 4, 5
 FP32_LANES_PER_SM = 128
 # the oracle's bounded sample: a centred window of the dominant eye
 ORACLE_WINDOW = (640, 480)
@@ -77,6 +78,7 @@ def parse():
     ap.add_argument("--warmup", type=int, default=4)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--n", type=int, default=500_000, help="surfels (default: the 500k workload)")
+    ap.add_argument("--detail", metavar="FILE", help="also write the whole record, unrounded, to FILE")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-learned", action="store_true",
                     help="skip training and timing the learned-repair variant")
@@ -102,6 +104,28 @@ def parse():
 
 def parse_raster(text):
     return None if text == "auto" else tuple(int(v) for v in text.split(","))
+
+
+def raster_kernel_name(cfg):
+    """The kernel a rasterizer configuration runs (8 of them serve the 28 configurations)."""
+    tile, pix, batch = cfg
+    stage = min(batch, 64)
+    return f"raster8_kernel<{pix}, {stage}>" if tile == 8 else f"raster16_kernel<{stage}>"
+
+
+# what the printed line leaves out, at any depth: lists per frame, timings of every
+# candidate, notes and splits
+DETAIL_KEYS = frozenset(("psnr_per_frame_db", "all_ms", "roi_tuning_ms", "per_step_ms", "note", "gain_bound", "training",
+                         "stage_ms", "stage_ms_stereo_plain", "timed_steps", "paths"))
+
+
+def brief(o):
+    """`o` with numbers to six significant digits and without the detail keys."""
+    if isinstance(o, dict):
+        return {k: brief(v) for k, v in o.items() if k not in DETAIL_KEYS}
+    if isinstance(o, (list, tuple)):
+        return [brief(v) for v in o]
+    return float(f"{o:.6g}") if isinstance(o, float) and math.isfinite(o) else o
 
 
 def dist_info():
@@ -671,19 +695,20 @@ def run_ours(args):
     hbm = float(pk["hbm_gbs"])
     peak_gops = sms * FP32_LANES_PER_SM * sm_mhz_peak * 1e6 / 1e9
     blend_ms = st_stereo[2]
-    pix = rc["stereo"][1]
+    pix = rc["stereo"][1] if rc["stereo"][0] == 8 else 2
     ops = OPS_PER_PAIR * float(np.mean(pairs_eval))
     own_ops = (OPS_EVAL_PIXEL + OPS_EVAL_COLUMN / pix) * float(np.mean(pairs_eval)) + \
         OPS_CONTRIB * float(np.mean(pairs_contrib))
     achieved = ops / (blend_ms * 1e-3) / 1e9
-    # dram read + write bytes of one ncu-captured launch of this blend kernel in
-    # this configuration ("traffic_bytes_per_launch <tile>x<pix>x<batch> = N" in
-    # a profiles/raster_*_object500k.md summary), or none
+    # dram read + write bytes of one ncu-captured launch of this blend kernel on
+    # the lists of this tile edge ("traffic_bytes_per_launch <kernel> tile <edge> = N"
+    # in a profiles/raster*_object500k.md summary), or none
     prof_traffic = None
-    key = "traffic_bytes_per_launch " + "x".join(map(str, rc["stereo"])) + " ="
+    blend_kernel = raster_kernel_name(rc["stereo"])
+    key = f"traffic_bytes_per_launch {blend_kernel} tile {rc['stereo'][0]} ="
     pdir = os.path.join(ROOT, "profiles")
     for name in sorted(os.listdir(pdir)) if os.path.isdir(pdir) else []:
-        if name.startswith("raster_") and name.endswith("_object500k.md"):
+        if name.startswith("raster") and name.endswith("_object500k.md"):
             for ln in open(os.path.join(pdir, name)):
                 if ln.startswith(key):
                     prof_traffic = int(ln.split("=")[1])
@@ -695,7 +720,7 @@ def run_ours(args):
                 "bytes": nbytes, "ms": ms, "work": unit_note, "peak_source": f"{pk_kind} copy bandwidth"}
 
     rooflines = {
-        "blend_dominant": {"bound": "alu", "kernel": "raster_kernel<" + ",".join(map(str, rc["stereo"])) + ">",
+        "blend_dominant": {"bound": "alu", "kernel": blend_kernel,
                            "achieved": achieved, "peak": peak_gops, "unit": "Gop/s", "frac": achieved / peak_gops,
                            "ms": blend_ms, "work": f"{OPS_PER_PAIR} ops x {np.mean(pairs_eval):.4g} evaluated pairs",
                            "own_count_frac": own_ops / (blend_ms * 1e-3) / 1e9 / peak_gops},
@@ -703,8 +728,10 @@ def run_ours(args):
                                PREPROCESS_BYTES_PER_SURFEL * scene.n, st_stereo[0],
                                f"{PREPROCESS_BYTES_PER_SURFEL} B x {scene.n} surfels"),
         "binning_dominant": hbm_line("dominant-eye binning (row spans, depth sort, row lists, "
-                                     "counting sort by tile)", BIN_BYTES_PER_INSTANCE * inst_dom, st_stereo[1],
-                                     f"{BIN_BYTES_PER_INSTANCE} B x {inst_dom:.4g} instances"),
+                                     "counting sort by tile; a chain bound by latency)",
+                                     BIN_BYTES_PER_SURFEL * scene.n + BIN_BYTES_PER_INSTANCE * inst_dom, st_stereo[1],
+                                     f"{BIN_BYTES_PER_SURFEL} B x {scene.n} surfels + {BIN_BYTES_PER_INSTANCE} B x "
+                                     f"{inst_dom:.4g} instances"),
         "warp_classify": hbm_line("warp, edge ROIs, gap classification", WARP_BYTES_PER_PIXEL * W * H, st_stereo[3],
                                   f"{WARP_BYTES_PER_PIXEL} B x {W * H} pixels"),
     }
@@ -786,7 +813,7 @@ def run_ours(args):
                    "stereo_roi": list(rc["roi"]) if rc["roi"] else "same as stereo",
                    "chosen_by": "autotuner" if tuning else "command line", "tuning": tuning,
                    "roi_tuning_ms": roi_tuning},
-        "roofline": {"bound": "alu", "kernel": "raster_kernel<" + ",".join(map(str, rc["stereo"])) + "> (dominant eye)",
+        "roofline": {"bound": "alu", "kernel": f"{blend_kernel} (dominant eye)",
                      "achieved": achieved, "peak": peak_gops,
                      "unit": "Gop/s", "frac": achieved / peak_gops, "traffic": prof_traffic,
                      "peak_source": f"{sms} SMs x 128 FP32 lanes x {sm_mhz_peak:.0f} MHz ({pk_kind} max clock)",
@@ -801,7 +828,10 @@ def run_ours(args):
         "backbone_3dgs": backbone3d,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.detail:
+            with open(args.detail, "w") as fh:
+                json.dump(line, fh)
+        print(json.dumps(brief(line)), flush=True)
     if ws_ > 1:
         torch.distributed.destroy_process_group()
 

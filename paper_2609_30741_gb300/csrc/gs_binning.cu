@@ -501,7 +501,8 @@ __device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
 // entries. A lane holds one surfel and its rows as a bit mask;
 // the transposed masks give every row's surfels, for the counts and the places.
 // Bound by the latency of the gathers in depth order (half of them miss L2 at 3M
-// surfels): six CTAs per SM (40 registers) measured 182 us there, four 199.
+// surfels at 2448x2448, dominant eye: 113 us; 182 with two ranges in 8 bytes a span and
+// 8-byte entries, with which four CTAs per SM instead of six took 199).
 __global__ void __launch_bounds__(kBinThreads, 6) row_list_kernel(ListArgs a) {
   griddep_wait();
   // per warp and row (padded to blocks of 32): pass 0 counts, then the warp's write
@@ -755,7 +756,8 @@ __global__ void __launch_bounds__(kBinThreads) bin_count_kernel(BinArgs a) {
 // per tile row: a whole band of four rows made a warp's chain of steps the time of
 // the launch. 1.5M / 3M surfels at 1920x1080 / 2448x2448: 44 / 105 us, against 94 /
 // 243 for an instance per lane ranked by shared-memory masks; collecting a CTA's
-// instances in shared memory for coalesced copies measured 53 / 112.
+// instances in shared memory for coalesced copies measured 53 / 112. All with the ids in
+// the entries; as gathers they cost 8 us more at 3M, and the row lists 69 less.
 // An entry's id is one more gather behind the entry: it goes to shared memory by
 // cp.async a step ahead, the first beside the counts' loads (loaded to a register with
 // the entry it cost 3 us of the 660 of the 500k-surfel frame).
