@@ -462,7 +462,8 @@ def run_ours(args):
         rc["roi"] = parse_raster(args.raster_roi)
     else:
         ctx.set_raster(*rc["stereo"])
-        cands = [None, (16, 2, 64), (16, 2, 128), (16, 4, 64), (16, 4, 128), (8, 2, 64), (32, 2, 64), (32, 2, 128)]
+        cands = [None, (16, 2, 32), (16, 2, 64), (8, 2, 64), (32, 2, 32), (32, 2, 64)]  # one per kernel worth a try
+        cands = [c for c in cands if c is None or (c[0], min(c[2], 64)) != (rc["stereo"][0], min(rc["stereo"][2], 64))]
         cands = [c for c in cands if c is None or c[0] >= ctx_min_tile]  # tiles the context can run
         evs = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(7)]
         for cand in cands:
