@@ -7,18 +7,20 @@
 // One CTA per 32 x 32 output tile and channel. Four quantities are filtered, as two
 // FP32x2 pairs: a = x + y and d = x - y, and their squares. With A, D their means and
 // va, vd their variances, 2 mx my = (A^2 - D^2) / 2, mx^2 + my^2 = (A^2 + D^2) / 2, and
-// likewise 2 sxy and sxx + syy from va and vd. For images that differ little (what a
-// quality metric is asked about) d is small and nearly exact, and the rounding of va,
-// which is that of squares near 4, enters numerator and denominator alike: flat white
-// with noise of 1e-4 is 1e-7 from the 64-bit value, and was 1e-5 from x^2 + y^2 and x y.
+// likewise 2 sxy and sxx + syy from va and vd. So the map's two factors are
+//   1 - 2 D^2 / (A^2 + D^2 + 2 C1)  and  1 - 2 vd / (va + vd + 2 C2),
+// and half of what their product lacks of 1 is summed. For images that differ little (what
+// a quality metric is asked about) that is small and nearly exact, while the rounding of
+// va, which is that of squares near 4, is in the denominator alone: flat white with noise
+// of 1e-4 is 3e-8 from the 64-bit value, and was 1e-5 from x^2 + y^2 and x y.
 // The 42 x 42 window of both images (zero outside)
 // goes to shared memory interleaved; a thread filters four columns of a row from
 // sixteen pixels in registers, and then eight rows of a column from eighteen
 // filtered rows, so an output costs four 16-byte shared-memory loads in place of
 // 77 4-byte ones. The map's sum is a double. FP64 runs at a fiftieth of
 // the FP32 rate here, so a thread first adds its eight values of a tile as an
-// unevaluated float pair (exact for values from 2^-19 to 2, within 2^-40 of smaller
-// ones) and then the pair to the double. The last CTA adds the partial sums in
+// unevaluated float pair (48 bits, exact for values within 2^20 of one another) and
+// then the pair to the double. The last CTA adds the partial sums in
 // a fixed order, so the result does not depend on scheduling.
 // 1919 x 1079 x 3: 56 us a call, bound by instruction issue; 94 for 4-byte loads, five
 // quantities, a double addition per value and a kernel to add the sums.
@@ -172,8 +174,8 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
     for (int o = 0; o < kSsRows; ++o) {
       if (ty0 + r0 + o >= H || tx0 + c >= W) continue;
       const float2 mm = __fmul2_rn(m[o], m[o]), vv = __ffma2_rn(make_float2(-m[o].x, -m[o].y), m[o], v[o]);
-      add_to(sum, err, ((mm.x - mm.y + 2.f * kC1) * (vv.x - vv.y + 2.f * kC2)) /
-                           ((mm.x + mm.y + 2.f * kC1) * (vv.x + vv.y + 2.f * kC2)));
+      const float dm = mm.x + mm.y + 2.f * kC1, dv = vv.x + vv.y + 2.f * kC2;
+      add_to(sum, err, fmaf(mm.y, dv, vv.y * (mm.x - mm.y + 2.f * kC1)) / (dm * dv));
     }
     total += (double)sum;
     if (isfinite(sum)) total += (double)err;  // of an infinite sum the error term is NaN
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(kSsThreads, kSsCtas) ssim_kernel(const float *
   for (uint32_t i = tid; i < gridDim.x; i += kSsThreads) t += __ldcg(part + i);
   t = block_sum(t, s_red);
   if (tid == 0) {
-    *out = (float)(t / count);
+    *out = (float)(1.0 - 2.0 * t / count);
     *ticket = 0u;  // for the next launch
   }
 }

@@ -38,3 +38,21 @@ def test_ssim_of_close_images(gs, shape, kind, noise):
     for p, q in ((a, b), (b, a)):
         assert abs(float(ctx.ssim(p, q)) - want) <= TOL, (float(ctx.ssim(p, q)), want)
     assert float(ctx.ssim(b, b)) == 1.0
+
+
+@pytest.mark.parametrize("noise", [1e-4, 1e-3])
+@pytest.mark.parametrize("shape", [(3, 37, 53), (3, 1199, 1599)])
+def test_ssim_next_to_one_is_rounded_once(gs, shape, noise):
+    """Uniform noise in [0, 1] and a copy with a little more: 1 - SSIM is below 1e-5, of
+    which 2^-16 is the most the filters' rounding makes (22 steps of 2^-24 on squares up to 4
+    against a variance of 0.3), and the result is rounded to a float once."""
+    from oracle import metrics
+    rng = np.random.default_rng(shape[2])
+    x = rng.random(shape)
+    y = x + noise * np.clip(rng.standard_normal(shape), -3.0, 3.0)
+    a, b = (torch.tensor(v, dtype=torch.float32, device="cuda") for v in (x, y))
+    ctx = gs.Context(16, 1600, 1200, max_instances=1 << 12)
+    want = metrics.ssim(a.double().cpu().numpy(), b.double().cpu().numpy())
+    assert 0.0 < 1.0 - want < 1e-5
+    for p, q in ((a, b), (b, a)):
+        assert abs(float(ctx.ssim(p, q)) - want) <= 2.0 ** -25 + 1e-5 * 2.0 ** -16
