@@ -56,3 +56,20 @@ def test_ssim_next_to_one_is_rounded_once(gs, shape, noise):
     assert 0.0 < 1.0 - want < 1e-5
     for p, q in ((a, b), (b, a)):
         assert abs(float(ctx.ssim(p, q)) - want) <= 2.0 ** -25 + 1e-5 * 2.0 ** -16
+
+
+@pytest.mark.parametrize("size", [(480, 640), (1079, 1919)])
+def test_window_weights_sum_to_one(gs, size):
+    """A smooth image and a noisy copy. A window that sums to 1 - e adds e A^2 to every
+    variance, 1.6e-7 of the SSIM for the weights' own rounding; without it what is left is
+    the result's rounding (2^-25) and the mean of the map's, far below as much again."""
+    from oracle import metrics
+    h, w = size
+    v, u = np.mgrid[:h, :w] / 24.0
+    rng = np.random.default_rng(h)
+    x = np.stack([0.5 + 0.2 * np.cos(u + c) + 0.2 * np.sin(0.7 * v - c) for c in range(3)])
+    y = x + 0.05 * rng.standard_normal(x.shape)
+    a, b = (torch.tensor(t, dtype=torch.float32, device="cuda") for t in (x, y))
+    ctx = gs.Context(16, w, h, max_instances=1 << 12)
+    want = metrics.ssim(a.double().cpu().numpy(), b.double().cpu().numpy())
+    assert abs(float(ctx.ssim(a, b)) - want) <= 2.0 ** -24, (float(ctx.ssim(a, b)), want)
